@@ -391,10 +391,12 @@ __device__ __forceinline__ void flush_keys(const uint2 *q, int n, uint32_t *s_lk
 // One CTA tile (rows by * 8 .. +7, columns bx * SPAN .. +SPAN-1) of one search:
 // the body of both the one-search kernel and the persistent batch kernel.
 // LONG: lists longer than kRankMax (walk insertion, predicated last load batch).
-// PRUNE: before a velocity's gathers, each warp adds its shifted span's bound
-// (one value per epoch from the span bound planes, kb_prune.cu: L2-resident, one
-// per 32 columns) and skips the velocity when the bound cannot reach nu_min^2
-// (the results do not change).
+// PRUNE: each warp adds its shifted span's bound (one value per epoch from the span
+// bound planes, kb_prune.cu: L2-resident, one per 32 columns) for 32 velocities at
+// once, a lane for each, and skips the velocities whose bound cannot reach nu_min^2
+// (the results do not change).  A velocity at a time (a lane for each epoch, then the
+// warp's sum) is a chain of a load and six shuffles for every velocity: 12 x 2048^2,
+// 1024 velocities, nu_min 10, psi/phi and bounds included: 8.72 ms that way, 4.10 this way.
 // KEYS: candidate lists in key form for the FP64 rescoring (a.cand_only, k <= kKeyMax).
 template <int STORAGE, int P, int C, bool LONG, typename I, bool PRUNE, bool KEYS = false>
 __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4) {
@@ -537,20 +539,31 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
         }
         __syncthreads();
         if (!active) continue;
+        unsigned todo = 0u;   // PRUNE: of the 32 velocities around vi, those to gather
         for (int vi = 0; vi < nc; ++vi) {
+            if constexpr (PRUNE) {
+                if ((vi & 31) == 0) {
+                    // a lane's velocity: its span's bound on nu^2, every step rounded upwards
+                    const int mine = vi + lane;
+                    float b = b0;
+                    if (mine < nc) {
+                        const E *t = s_tab + mine * NJP;
+                        const I *rid = s_rid + mine * NJP;
+#pragma unroll 4
+                        for (int jj = 0; jj < NJ; ++jj)
+                            if (t[jj].info & wbit) b = __fadd_ru(b, __ldg(a.snr2 + rid[jj] + (long long)warp * RW));
+                    }
+                    todo = __ballot_sync(0xffffffffu, mine < nc && !(__fmul_ru(b, 1.0f + 0x1p-14f) < a.nu_min2_slack));
+                }
+                const unsigned rest = todo >> (vi & 31);
+                if (rest == 0u) {
+                    vi |= 31;
+                    continue;
+                }
+                vi += __ffs(rest) - 1;
+            }
             const int v = s_vid[vi];
             const E *tab = s_tab + vi * NJP;
-            if constexpr (PRUNE) {
-                // the span's bound on nu^2, rounded upwards, lane 0's sum for the whole warp
-                float b = 0.0f;
-                const I *rid = s_rid + vi * NJP;
-                for (int jj = lane; jj < NJ; jj += 32)
-                    if (tab[jj].info & wbit) b = __fadd_ru(b, __ldg(a.snr2 + rid[jj] + (long long)warp * RW));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) b = __fadd_ru(b, __shfl_xor_sync(0xffffffffu, b, o));
-                b = __shfl_sync(0xffffffffu, b, 0);
-                if (__fmul_ru(__fadd_ru(b, b0), 1.0f + 0x1p-14f) < a.nu_min2_slack) continue;
-            }
             float2 acc[PX];
 #pragma unroll
             for (int p = 0; p < PX; ++p) acc[p] = acc0[p];
