@@ -993,10 +993,7 @@ struct kb_batch {
 
 namespace {
 
-int index_bits(const kb::SearchArgs &a) {
-    const long long span = (a.storage == KB_F32 ? 1LL : 2LL) * a.N * a.plane_elems;
-    return span < (1LL << 31) - 1 ? 32 : 64;
-}
+int index_bits(const kb::SearchArgs &a) { return kb::search_idx32(a) ? 32 : 64; }
 
 // Items of a group for one tile shape: whole searches, or (sample) a band of
 // about `frac` of each search's rows from its middle.

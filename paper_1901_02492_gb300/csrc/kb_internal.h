@@ -223,8 +223,41 @@ struct SearchArgs {
     const float *snr2;       // KB_PRUNE: span bound planes [N][H][(W + 31) / 32 + span / 32] (stack epochs), else null
     float nu_min2_slack;     // KB_PRUNE: skip a span when its bound times (1 + 2^-14) is below this (nu_min^2)
 };
+// whether the search addresses the planes (both phases) by 32-bit byte offsets
+inline bool search_idx32(const SearchArgs &a) {
+    return a.planes_elems * (a.storage == KB_F32 ? (long long)sizeof(float2) : (long long)sizeof(pair16)) < (1LL << 32);
+}
 // register-gather kernel (variant 0 = its default shape, 1..4)
 cudaError_t launch_search(const SearchArgs &a, cudaStream_t st);
+// one storage's kernels (kb_search.cu, kb_search_bf16.cu, kb_search_f16.cu)
+template <int STORAGE>
+cudaError_t launch_search_storage(const SearchArgs &a, cudaStream_t st);
+template <int STORAGE>
+cudaError_t launch_search_batch_storage(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int variant,
+                                        int kmax, int carve, bool idx64, int sm_count, cudaStream_t st);
+template <int STORAGE>
+cudaError_t debug_word_storage(unsigned long long *word, bool reset);
+template <>
+cudaError_t launch_search_storage<KB_F32>(const SearchArgs &, cudaStream_t);
+template <>
+cudaError_t launch_search_batch_storage<KB_F32>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+                                               cudaStream_t);
+template <>
+cudaError_t debug_word_storage<KB_F32>(unsigned long long *, bool);
+template <>
+cudaError_t launch_search_storage<KB_BF16>(const SearchArgs &, cudaStream_t);
+template <>
+cudaError_t launch_search_batch_storage<KB_BF16>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+                                               cudaStream_t);
+template <>
+cudaError_t debug_word_storage<KB_BF16>(unsigned long long *, bool);
+template <>
+cudaError_t launch_search_storage<KB_F16>(const SearchArgs &, cudaStream_t);
+template <>
+cudaError_t launch_search_batch_storage<KB_F16>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+                                               cudaStream_t);
+template <>
+cudaError_t debug_word_storage<KB_F16>(unsigned long long *, bool);
 // KB_DEBUG builds: the first out-of-bounds access the search kernels recorded
 // ((site << 56) | offset, 0 if none), then cleared if reset; cudaErrorNotSupported
 // in other builds

@@ -13,19 +13,17 @@
 //     one plane row: fully coalesced 8-byte loads.  16-bit pairs are 8-byte
 //     aligned because the planes also exist shifted by one pixel (the "phase 1"
 //     copy) and odd shifts read that copy;
-//   - the (velocity, epoch) table is staged per CTA in shared memory and checked
-//     there once: each entry holds the element offset of the shifted row start
-//     (epoch plane and phase included), a mask of the CTA's warps whose shifted
-//     span overlaps the image, and for 16-bit storage the epoch's two
-//     power-of-two scales as bf16 bit patterns (the FMA's scale operand).  The
-//     inner loop per entry is one broadcast load, one mask test selecting the
-//     entry's offset or the offset of a zero block, one wide multiply-add for
-//     the address, the gathers and one packed f32x2 add per pixel (16-bit: one
-//     mixed-precision FMA per value);
-//   - spans that overlap the image only partly read the zero columns the planes
-//     carry left and right of every row (kSpan wide); spans that miss it read the
-//     zero columns left of row 0 of plane 0, which stay in L1, so off-image steps
-//     cost no memory traffic and "outside contributes nothing" holds exactly;
+//   - the (velocity, epoch) table is staged per CTA in shared memory, a row per velocity:
+//     one entry for each epoch whose shifted band (8 rows x SPAN columns) overlaps the
+//     image, in time order, holding the offset of the shifted row start (epoch plane and
+//     phase included) and for 16-bit storage the epoch's two power-of-two scales as bf16
+//     bit patterns (the FMA's scale operand).  Epochs that miss the image are left out:
+//     they add nothing.  Entries are read four to a group of 16-byte broadcast loads; per
+//     entry and load there is an address, the gather and one packed f32x2 add per pixel
+//     (16-bit: one mixed-precision FMA per value);
+//   - bands that overlap the image only partly read the zero columns the planes carry left
+//     and right of every row (kSpan wide) and the zero rows above and below every plane
+//     (kPadRows), so "outside contributes nothing" holds exactly without a bounds check;
 //   - epochs at t = t_min have offset 0 for every velocity: their contribution is
 //     loaded once per pixel before the velocity loop;
 //   - velocities are processed in the order the host planner gives (sorted by
@@ -35,51 +33,36 @@
 //   - CTAs take their tiles in super-columns a few tiles wide, row by row within
 //     each, so the CTAs resident at one time cover a compact block of start
 //     pixels and the late epochs' rows they read stay in L2;
-//   - top-k: each pixel's list of (nu, 16-bit velocity index), best first, is in
-//     shared memory (slot-major: slot i of list column c at c + i * LS, so the
-//     lanes of a warp touch distinct banks); the k-th entry is mirrored in
-//     registers as the admission threshold.  A trajectory that beats its pixel's
-//     threshold is not inserted at once: the warp appends it to a queue in
-//     shared memory (ballot + popc), and when 32 or more are pending every lane
-//     inserts one.  Candidates arrive at scattered velocities for the 64-128
-//     pixels of a warp, so inserting on arrival keeps the warp busy for one
-//     lane's insertion at almost every velocity; batched, the lanes insert
-//     together.  Lists up to 8 long insert by rank (all slots loaded at once,
-//     then the tail shifted); longer ones walk up from the last slot.
+//   - top-k: each pixel's list of (nu, 16-bit velocity index), best first, and a short
+//     buffer of new entries are in shared memory (slot-major: slot i of list column c at
+//     c + i * LS, so the lanes of a warp touch distinct banks); the k-th entry is mirrored
+//     in registers as the admission threshold.  A trajectory that beats its pixel's
+//     threshold is appended to the buffer by its own lane, and when one of a warp's
+//     buffers is full, all its lanes merge theirs in lock step.
 // The Psi/Phi of each kept trajectory are recomputed at the end by the same
 // sequence of operations (bit-identical) together with nobs.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
+#include <string.h>
 
 #include "kb_device.cuh"
 
+// This file compiles one storage's kernels: FP32's and the common entry points by itself,
+// the 16-bit ones when kb_search_bf16.cu and kb_search_f16.cu include it (three translation
+// units that build side by side).
+#ifndef KB_SEARCH_STORAGE
+#define KB_SEARCH_STORAGE KB_F32
+#define KB_SEARCH_COMMON
+#endif
+
 namespace kb {
-
-#ifdef KB_DEBUG
-// KB_DEBUG: the first out-of-bounds access of the search kernels, (site << 56) | offset
-__device__ unsigned long long g_debug_word;
-#endif
-
-cudaError_t debug_word(unsigned long long *word, bool reset) {
-#ifdef KB_DEBUG
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = cudaMemcpyFromSymbol(word, g_debug_word, sizeof(*word));
-    if (e == cudaSuccess && reset) {
-        const unsigned long long zero = 0;
-        e = cudaMemcpyToSymbol(g_debug_word, &zero, sizeof(zero));
-    }
-    return e;
-#else
-    (void)word;
-    (void)reset;
-    return cudaErrorNotSupported;
-#endif
-}
 
 namespace {
 
 #ifdef KB_DEBUG
+// KB_DEBUG: the first out-of-bounds access of this storage's kernels, (site << 56) | offset
+__device__ unsigned long long g_debug_word;
 __device__ __noinline__ void debug_record(int site, long long at) {
     atomicCAS(&g_debug_word, 0ull, ((unsigned long long)site << 56) | ((unsigned long long)at & 0x00ffffffffffffffull));
 }
@@ -124,12 +107,9 @@ using namespace dev;
 constexpr int WARPS = 8;
 constexpr int THREADS = WARPS * 32;
 constexpr uint16_t kNoV = 0xFFFF;   // empty list slot (velocity indices are < 65535)
-constexpr int kRankMax = 8;         // lists up to this long insert by rank, longer ones by walking
-
-// (velocity, epoch) entries staged per chunk (small: occupancy); the 16-bit
-// entries are twice as large and their CTAs hold twice the pixels
-template <int STORAGE>
-__host__ __device__ constexpr int tab_entries() { return STORAGE == KB_F32 ? 512 : 256; }
+constexpr int kShortMax = 8;        // lists up to this long merge in a network of 8,
+constexpr int kKeyMax = 16;         // up to this (and key lists) in one of 16,
+constexpr int kListMax = 32;        // and all others by walking
 
 __device__ __forceinline__ float2 exp_scale(int e) {
     return make_float2(__int_as_float((e & 0xff) << 23), __int_as_float(((e >> 8) & 0xff) << 23));
@@ -186,144 +166,71 @@ struct Gather<KB_F16> {
     }
 };
 
-// staged table entry: element offset (32 or 64 bit), the mask of the CTA's warps
-// whose shifted span overlaps the image, and for 16-bit storage the epoch's scale
-// operand (16 bytes: one shared load)
+// Staged table entry: the shifted row start of one (velocity, epoch), relative to the
+// lane's place in plane 0 (LaneBase), and for 16-bit storage (SC) the epoch's scale operand.
 template <typename I, bool SC>
 struct Entry;
 template <typename I>
 struct Entry<I, false> {
     I idx;
-    int info;
 };
-template <>
-struct Entry<int, true> {
-    int idx;
-    int info;
-    uint32_t sc, pad;
-};
-template <>
-struct Entry<long long, true> {
-    long long idx;
-    int info;
+template <typename I>
+struct Entry<I, true> {
+    I idx;
     uint32_t sc;
 };
-// FP32 planes, 32-bit offsets, no pruning: compact 4-byte entries (search_tile), twice as
-// many per chunk of the table in the same shared bytes
-template <int STORAGE, typename I, bool PRUNE>
-__host__ __device__ constexpr bool compact_entries() { return STORAGE == KB_F32 && sizeof(I) == 4 && !PRUNE; }
+// Bytes of entries per chunk of the table.  A velocity's row is a whole number of groups of
+// four entries, so a chunk holds at most a quarter as many velocities as entries.  FP32: 2 KB
+// (42 velocities of 11 epochs), which with buffers of 4 leaves 4 CTAs per SM within the
+// 164 KB shared-memory split and 92 KB to L1 (12 x 4096^2, k = 8: 75.8 ms; 4 KB: 78.1); the
+// pruned search, which takes bounds for 32 velocities of a chunk at once, 4 KB (12 x 2048^2,
+// nu_min 10: 3.68 ms; 2 KB: 3.95).  16-bit: 4 KB.
+template <int STORAGE, typename I>
+__host__ __device__ constexpr size_t table_entry_bytes() { return sizeof(Entry<I, STORAGE != KB_F32>); }
 template <int STORAGE, typename I, bool PRUNE>
 __host__ __device__ constexpr int table_entries() {
-    return compact_entries<STORAGE, I, PRUNE>() ? 2 * tab_entries<STORAGE>() : tab_entries<STORAGE>();
-}
-template <int STORAGE, typename I, bool PRUNE>
-__host__ __device__ constexpr size_t table_entry_bytes() {
-    return compact_entries<STORAGE, I, PRUNE>() ? sizeof(int) : sizeof(Entry<I, STORAGE != KB_F32>);
+    return (int)((STORAGE == KB_F32 && !PRUNE ? 2048 : 4096) / table_entry_bytes<STORAGE, I>());
 }
 template <typename I>
 __device__ __forceinline__ uint32_t entry_sc(const Entry<I, false> &) { return 0u; }
 template <typename I>
 __device__ __forceinline__ uint32_t entry_sc(const Entry<I, true> &e) { return e.sc; }
 
-// two consecutive table entries (the first at an even index) in one 16-byte load
+// four consecutive table entries, the first at a multiple of four, in 16-byte loads
 template <typename E>
-__device__ __forceinline__ void load_pair(const E *t, E &a, E &b) {
-    if constexpr (sizeof(E) == 8) {
-        const int4 w = *reinterpret_cast<const int4 *>(t);
-        a.idx = w.x;
-        a.info = w.y;
-        b.idx = w.z;
-        b.info = w.w;
-    } else {
-        a = t[0];
-        b = t[1];
-    }
+__device__ __forceinline__ void load_four(const E *t, E (&e)[4]) {
+    static_assert(sizeof(E) % 4 == 0 && sizeof(E) <= 16, "a group of four entries is a whole number of 16-byte words");
+    int4 w[sizeof(E) / 4];
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(E) / 4); ++i) w[i] = reinterpret_cast<const int4 *>(t)[i];
+    memcpy(e, w, sizeof e);
 }
 
-// Insert (cn, cv) into the list of column `col` (slot i at col + i * LS), if it
-// beats the list's last entry.  Lists up to kRankMax long: every slot is loaded
-// at once, the candidate's rank is the number of entries better than it, and the
-// entries below it move down one slot.  Longer lists: a walk up from the last slot.
-template <bool LONG>
-__device__ __forceinline__ void list_insert(float *s_ln, uint16_t *s_lv, int col, int k, int LS, float cn, int cv) {
-    float *ln = s_ln + col;
-    uint16_t *lv = s_lv + col;
-    if constexpr (!LONG) {
-        float en[kRankMax];
-        int ev[kRankMax];
-        int pos = 0;
-#pragma unroll
-        for (int i = 0; i < kRankMax; ++i) {
-            en[i] = -INFINITY;
-            ev[i] = kNoV;
-            if (i < k) {
-                en[i] = ln[i * LS];
-                ev[i] = lv[i * LS];
-            }
-            pos += (i < k && better(en[i], ev[i], cn, cv)) ? 1 : 0;
-        }
-        if (pos < k) {
-#pragma unroll
-            for (int i = kRankMax - 1; i > 0; --i)
-                if (i < k && i > pos) {
-                    ln[i * LS] = en[i - 1];
-                    lv[i * LS] = (uint16_t)ev[i - 1];
-                }
-            ln[pos * LS] = cn;
-            lv[pos * LS] = (uint16_t)cv;
-        }
-    } else {
-        int i = k - 1;
-        if (!better(cn, cv, ln[i * LS], lv[i * LS])) return;
-        while (i > 0) {
-            const float pn = ln[(i - 1) * LS];
-            const int pv = lv[(i - 1) * LS];
-            if (!better(cn, cv, pn, pv)) break;
-            ln[i * LS] = pn;
-            lv[i * LS] = (uint16_t)pv;
-            --i;
-        }
-        ln[i * LS] = cn;
-        lv[i * LS] = (uint16_t)cv;
+// A lane's place in the planes, and where its loads of an entry start.  BYTES: a 32-bit byte
+// offset from the planes' base, to which the entry's is added modulo 2^32 -- one register
+// instead of a pointer's two; else a pointer.
+template <typename T, bool BYTES>
+struct LaneBase {
+    const T *p;
+    __device__ __forceinline__ LaneBase(const T *planes, long long elem) : p(planes + elem) {}
+    template <typename I>
+    __device__ __forceinline__ const T *at(const T *, I idx) const { return p + idx; }
+    __device__ __forceinline__ static long long offset(long long elem) { return elem; }
+};
+template <typename T>
+struct LaneBase<T, true> {
+    uint32_t b;
+    __device__ __forceinline__ LaneBase(const T *, long long elem) : b(offset(elem)) {}
+    __device__ __forceinline__ const T *at(const T *planes, int idx) const {
+        return reinterpret_cast<const T *>(reinterpret_cast<const char *>(planes) + ((uint32_t)idx + b));
     }
-}
-
-// Insert the warp's n pending candidates {nu bits, vidx | (p * 32 + lane) << 16}
-// into their pixels' lists, then reload every lane's register thresholds.  Each
-// round takes 32 entries, one per lane; entries of one pixel are inserted one
-// after the other (match_any groups them), so a list is written by one lane at a
-// time.  A candidate that no longer beats its list's last entry is dropped.  The
-// result does not depend on the order of insertion: a list ends as the k best of
-// everything offered to it under (nu desc, vidx asc).
-template <int PX, bool LONG>
-__device__ __forceinline__ void flush_queue(const uint2 *q, int n, float *s_ln, uint16_t *s_lv, int k, int LS,
-                                            int warp, int lane, float *thn, int *thv) {
-    for (int b = 0; b < n; b += 32) {
-        bool pend = b + lane < n;
-        uint2 e = make_uint2(0u, 0u);
-        if (pend) e = q[b + lane];
-        const float cn = __uint_as_float(e.x);
-        const int cv = (int)(e.y & 0xffffu);
-        const int pc = (int)(e.y >> 16);
-        const int col = (pc >> 5) * THREADS + warp * 32 + (pc & 31);
-        // at most 32 sub-rounds: each inserts at least the lowest pending lane of every group
-        for (;;) {
-            if (!__any_sync(0xffffffffu, pend)) break;
-            const unsigned grp = __match_any_sync(0xffffffffu, pend ? pc : 256 + lane);
-            if (pend && lane == __ffs(grp) - 1) {
-                pend = false;
-                if (debug_in(col, LS, 6)) list_insert<LONG>(s_ln, s_lv, col, k, LS, cn, cv);
-            }
-            __syncwarp();
-        }
-    }
-#pragma unroll
-    for (int p = 0; p < PX; ++p) {
-        const int c = p * THREADS + warp * 32 + lane;
-        thn[p] = s_ln[c + (k - 1) * LS];
-        thv[p] = s_lv[c + (k - 1) * LS];
-    }
-}
+    __device__ __forceinline__ static uint32_t offset(long long elem) { return (uint32_t)(elem * (long long)sizeof(T)); }
+};
+// Byte offsets where registers are short: FP32 lists up to 8 long, held to 64 (12 x 4096^2,
+// k = 8: 75.8 ms; pointers 80.5, one value of the loop in local memory).  Elsewhere the
+// extra add costs more: BF16 key lists 25.8 ms against 25.5 with pointers (4096 x 2048).
+template <int STORAGE, int KM, bool KEYS, typename I>
+__host__ __device__ constexpr bool byte_offsets() { return sizeof(I) == 4 && STORAGE == KB_F32 && KM <= kShortMax; }
 
 // Candidate lists of a search that only feeds the FP64 rescoring (KEYS): one
 // 32-bit key per slot.  With b = a.key_bits bits for a velocity index, the high
@@ -337,8 +244,6 @@ __device__ __forceinline__ void flush_queue(const uint2 *q, int n, float *s_ln, 
 // value).  A key's value hi and the value lo one step of 2^b below it in the
 // encoding bracket the unrounded nu: lo < nu <= hi.  Empty slots are key 0, below
 // the key of every finite nu (whose encoding is at least 2^23).
-constexpr int kKeyMax = 16;   // longest candidate list in key form
-
 __device__ __forceinline__ uint32_t nu_key(float nu, int v, int b) {
     const uint32_t u = __float_as_uint(nu), m = (1u << b) - 1u;
     const uint32_t ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
@@ -346,51 +251,190 @@ __device__ __forceinline__ uint32_t nu_key(float nu, int v, int b) {
     return (q << b) | (m - (uint32_t)v);
 }
 
-// Rank insertion of key ck into the key list of column `col` (k <= kKeyMax slots,
-// best first), if it beats the list's last entry.
-__device__ __forceinline__ void key_insert(uint32_t *s_lk, int col, int k, int LS, uint32_t ck) {
-    uint32_t *lk = s_lk + col;
-    if (!(ck > lk[(k - 1) * LS])) return;
-    uint32_t e[kKeyMax];
-    int pos = 0;
-#pragma unroll
-    for (int i = 0; i < kKeyMax; ++i) {
-        e[i] = i < k ? lk[i * LS] : 0u;
-        pos += (i < k && e[i] > ck) ? 1 : 0;
-    }
-#pragma unroll
-    for (int i = kKeyMax - 1; i > 0; --i)
-        if (i < k && i > pos) lk[i * LS] = e[i - 1];
-    lk[pos * LS] = ck;
+// ---- per-pixel top-k lists ------------------------------------------------------
+// A list column (one pixel, owned by one lane) holds its k best entries, sorted, then a
+// buffer of CAP entries.  A trajectory that beats the pixel's threshold (its k-th entry
+// at the last merge) is appended to the buffer by its own lane, without a vote or a
+// conflict; when one of the warp's buffers is full, every lane merges its own buffers
+// into its lists in registers, in lock step, with a sorting network.  A pixel admits about
+// k (1 + log(V / k)) entries, 47 of 1024 velocities at k = 8, and a merge costs the same
+// for one new entry as for CAP.  A queue common to the warp, emptied 32 entries at a time
+// with a rank insertion each (match, ranks, bank conflicts between the pixels of a round),
+// executed 17.9 G warp instructions and 1.43 G shared wavefronts at 12 x 2048^2, k = 8,
+// against 15.2 G and 0.95 G (and 16.6 G with the queue and the same table).  The result
+// does not depend on the order of arrival: a list ends as the k best of everything offered
+// to it under (nu desc, vidx asc).
+
+// an entry as one ordered word: nu's order-preserving encoding above 0xffff - vidx
+__device__ __forceinline__ unsigned long long slot_key(float nu, int v) {
+    const uint32_t u = __float_as_uint(nu + 0.0f);   // -0 and +0 are one score
+    const uint32_t ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return ((unsigned long long)ord << 32) | (0xffffu - (uint32_t)v);
+}
+__device__ __forceinline__ float slot_nu(unsigned long long key) {
+    const uint32_t ord = (uint32_t)(key >> 32);
+    return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7FFFFFFFu) : ~ord);
+}
+__device__ __forceinline__ int slot_vidx(unsigned long long key) { return (int)(0xffffu - (uint32_t)(key & 0xffffu)); }
+
+template <typename K>
+__device__ __forceinline__ void order_desc(K &a, K &b) {
+    const K hi = a > b ? a : b, lo = a > b ? b : a;
+    a = hi;
+    b = lo;
 }
 
-// flush_queue for key lists: entries {key, (p * 32 + lane) << 16}
-template <int PX>
-__device__ __forceinline__ void flush_keys(const uint2 *q, int n, uint32_t *s_lk, int k, int LS, int warp, int lane,
-                                           uint32_t *thk) {
-    for (int b = 0; b < n; b += 32) {
-        bool pend = b + lane < n;
-        uint2 e = make_uint2(0u, 0u);
-        if (pend) e = q[b + lane];
-        const int pc = (int)(e.y >> 16);
-        const int col = (pc >> 5) * THREADS + warp * 32 + (pc & 31);
-        for (;;) {   // at most 32 sub-rounds, as in flush_queue
-            if (!__any_sync(0xffffffffu, pend)) break;
-            const unsigned grp = __match_any_sync(0xffffffffu, pend ? pc : 256 + lane);
-            if (pend && lane == __ffs(grp) - 1) {
-                pend = false;
-                if (debug_in(col, LS, 6)) key_insert(s_lk, col, k, LS, e.x);
+// the list l (KM entries, sorted, best first) becomes the KM best of itself and b (CAP <= KM
+// entries in any order): b is sorted by Batcher's odd-even merge network, its reverse
+// compared with the tail of l, and the bitonic sequence this leaves is merged
+template <int KM, int CAP, typename K>
+__device__ __forceinline__ void merge_best(K (&l)[KM], K (&b)[CAP]) {
+#pragma unroll
+    for (int p = 1; p < CAP; p *= 2) {
+#pragma unroll
+        for (int q = p; q >= 1; q /= 2) {
+#pragma unroll
+            for (int j = q % p; j + q < CAP; j += 2 * q) {
+#pragma unroll
+                for (int i = 0; i < q; ++i)
+                    if (i + j + q < CAP && (i + j) / (2 * p) == (i + j + q) / (2 * p)) order_desc(b[i + j], b[i + j + q]);
             }
-            __syncwarp();
         }
     }
 #pragma unroll
-    for (int p = 0; p < PX; ++p) thk[p] = s_lk[p * THREADS + warp * 32 + lane + (k - 1) * LS];
+    for (int i = 0; i < CAP; ++i) l[KM - 1 - i] = l[KM - 1 - i] > b[i] ? l[KM - 1 - i] : b[i];
+#pragma unroll
+    for (int h = KM / 2; h >= 1; h /= 2) {
+#pragma unroll
+        for (int i = 0; i < KM; ++i)
+            if ((i & h) == 0) order_desc(l[i], l[i + h]);
+    }
+}
+
+// Merges the n buffered entries of a column into its list of k and sets its threshold, the
+// list's k-th entry; slot i lies at i * LS of ln and lv (value lists) or lk (key lists).
+// Inlined: as calls they cost the longer lists 8 % and more (2111 x 2045, 14 epochs, k = 12:
+// 18.4 ms against 16.6; BF16 key lists, 4096 x 2048: 27.6 against 25.5).
+template <int KM, int CAP, int LS>
+__device__ __forceinline__ void merge_values(float *ln, uint16_t *lv, int k, int n, float &thn, int &thv) {
+    unsigned long long l[KM], b[CAP];
+#pragma unroll
+    for (int i = 0; i < KM; ++i) l[i] = i < k ? slot_key(ln[i * LS], lv[i * LS]) : 0ull;
+#pragma unroll
+    for (int i = 0; i < CAP; ++i) b[i] = i < n ? slot_key(ln[(k + i) * LS], lv[(k + i) * LS]) : 0ull;
+    merge_best<KM, CAP>(l, b);
+#pragma unroll
+    for (int i = 0; i < KM; ++i) {
+        if (i < k) {
+            ln[i * LS] = slot_nu(l[i]);
+            lv[i * LS] = (uint16_t)slot_vidx(l[i]);
+        }
+    }
+    thn = ln[(k - 1) * LS];
+    thv = lv[(k - 1) * LS];
+}
+template <int KM, int CAP, int LS>
+__device__ __forceinline__ void merge_keys(uint32_t *lk, int k, int n, uint32_t &thk) {
+    uint32_t l[KM], b[CAP];
+#pragma unroll
+    for (int i = 0; i < KM; ++i) l[i] = i < k ? lk[i * LS] : 0u;
+#pragma unroll
+    for (int i = 0; i < CAP; ++i) b[i] = i < n ? lk[(k + i) * LS] : 0u;
+    merge_best<KM, CAP>(l, b);
+#pragma unroll
+    for (int i = 0; i < KM; ++i)
+        if (i < k) lk[i * LS] = l[i];
+    thk = lk[(k - 1) * LS];
+}
+
+// Lists of 17 to 24 (only wide rescoring searches keep them): each buffered entry walks up from
+// the last slot.  A network of 32 inlined would crowd out the search's loop.
+template <int LS>
+__device__ __forceinline__ void insert_values(float *ln, uint16_t *lv, int k, int n, float &thn, int &thv) {
+    for (int e = 0; e < n; ++e) {
+        const float cn = ln[(k + e) * LS];
+        const int cv = lv[(k + e) * LS];
+        int i = k - 1;
+        if (!better(cn, cv, ln[i * LS], lv[i * LS])) continue;
+        while (i > 0) {
+            const float pn = ln[(i - 1) * LS];
+            const int pv = lv[(i - 1) * LS];
+            if (!better(cn, cv, pn, pv)) break;
+            ln[i * LS] = pn;
+            lv[i * LS] = (uint16_t)pv;
+            --i;
+        }
+        ln[i * LS] = cn;
+        lv[i * LS] = (uint16_t)cv;
+    }
+    thn = ln[(k - 1) * LS];
+    thv = lv[(k - 1) * LS];
+}
+
+// Buffer entries of a column.  More of them mean fewer merges but a larger shared-memory
+// footprint, and what the lists take the L1 loses: 12 x 4096^2, k = 8, FP32: 3 entries
+// 80.0 ms, 4 75.8, 6 83.4; 2111 x 2045, 14 epochs, k = 12: 3 18.0 ms, 4 16.9, 5 16.6, 6 17.1;
+// key lists (4096 x 2048 BF16, k_c = 12, with the rescoring): 3 26.1 ms, 4 25.5, 5 25.8.
+// Value lists of four pixels per lane: 3, so that at k = 8 the 1024-pixel CTAs' lists leave room
+// for 3 CTAs per SM (FP16, 1500 x 1700, 10 epochs, 500 velocities: (2, 4) 7.52 ms; 4 entries 7.98).
+template <int KM, bool KEYS, int PX>
+__host__ __device__ constexpr int list_cap() { return KEYS ? 4 : KM > kShortMax ? 5 : PX == 4 ? 3 : 4; }
+
+// Adds B epochs (a multiple of four) of one velocity to a lane's sums: every load issued
+// before the first sum, the sums in epoch order.
+template <int STORAGE, int P, int B, typename E, typename T, typename L>
+__device__ __forceinline__ void add_epochs(const E *tab, const L &lane0, const T *planes, long long elems, float2 *acc) {
+    typedef Gather<STORAGE> G;
+    typedef typename G::LT LT;
+    LT val[B][P];
+    uint32_t sc[B];
+#pragma unroll
+    for (int q = 0; q < B; q += 4) {
+        E e[4];
+        load_four(tab + q, e);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            sc[q + h] = entry_sc(e[h]);
+            const LT *src = reinterpret_cast<const LT *>(lane0.at(planes, e[h].idx));
+#pragma unroll
+            for (int p = 0; p < P; ++p) val[q + h][p] = gather(src + 32 * p, planes, elems, 2);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[q][p], sc[q]);
+    }
+}
+
+// The last 1 to 3 epochs of a velocity (n is the same for the whole warp)
+template <int STORAGE, int P, typename E, typename T, typename L>
+__device__ __forceinline__ void add_tail(const E *tab, int n, const L &lane0, const T *planes, long long elems, float2 *acc) {
+    typedef Gather<STORAGE> G;
+    typedef typename G::LT LT;
+    E e[4];
+    load_four(tab, e);   // the row's padding included, unused
+    LT val[3][P];
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+        if (h < n) {
+            const LT *src = reinterpret_cast<const LT *>(lane0.at(planes, e[h].idx));
+#pragma unroll
+            for (int p = 0; p < P; ++p) val[h][p] = gather(src + 32 * p, planes, elems, 3);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+        if (h < n) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[h][p], entry_sc(e[h]));
+        }
+    }
 }
 
 // One CTA tile (rows by * 8 .. +7, columns bx * SPAN .. +SPAN-1) of one search:
 // the body of both the one-search kernel and the persistent batch kernel.
-// LONG: lists longer than kRankMax (walk insertion, predicated last load batch).
+// KM: the lists' longest length, which says how they merge.
 // PRUNE: each warp adds its shifted span's bound (one value per epoch from the span
 // bound planes, kb_prune.cu: L2-resident, one per 32 columns) for 32 velocities at
 // once, a lane for each, and skips the velocities whose bound cannot reach nu_min^2
@@ -398,46 +442,33 @@ __device__ __forceinline__ void flush_keys(const uint2 *q, int n, uint32_t *s_lk
 // warp's sum) is a chain of a load and six shuffles for every velocity: 12 x 2048^2,
 // 1024 velocities, nu_min 10, psi/phi and bounds included: 8.72 ms that way, 4.10 this way.
 // KEYS: candidate lists in key form for the FP64 rescoring (a.cand_only, k <= kKeyMax).
-template <int STORAGE, int P, int C, bool LONG, typename I, bool PRUNE, bool KEYS = false>
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false>
 __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4) {
     typedef Store<STORAGE> St;
     typedef typename St::T T;         // one pixel's (psi, phi)
     typedef Gather<STORAGE> G;
     typedef typename G::LT LT;        // one load
     typedef Entry<I, STORAGE != KB_F32> E;
-    // Compact entries (FP32 planes, 32-bit offsets, no pruning): one 4-byte offset per
-    // (velocity, epoch), four to a 16-byte shared load.  The planes' zero rows above and
-    // below make every warp's row of a band that overlaps the image's rows valid, so no
-    // per-warp mask is needed; a band that misses the image gets the offset of the CTA's
-    // rows of zeros above row 0 of plane 0 (any warp lands in them).
-    constexpr bool CE = compact_entries<STORAGE, I, PRUNE>();
-    static_assert(!CE || C % 4 == 0, "compact entries are read four at a time");
+    static_assert(C % 4 == 0, "entries are read four at a time");
     static_assert(WARPS <= kPadRows, "a band of warps' rows must fit the planes' zero rows");
-    constexpr int TAB = table_entries<STORAGE, I, PRUNE>();
-    constexpr size_t EB = table_entry_bytes<STORAGE, I, PRUNE>();
+    constexpr int TAB = table_entries<STORAGE, I, PRUNE>(), ROWS = TAB / 4;
+    constexpr size_t EB = table_entry_bytes<STORAGE, I>();
     constexpr int PX = P * G::PIX;    // pixels per lane
     constexpr int SPAN = 32 * PX;     // pixels per warp row segment
     constexpr int LS = THREADS * PX;  // list columns (pixels) of the CTA
-    constexpr int QCAP = 32 * (PX + 1);   // < 32 pending after a flush, + one velocity's candidates
+    constexpr int CAP = list_cap<KM, KEYS, PX>();             // buffer entries of a column
 
     // s_scale: per time-ordered epoch.  s_dyn4: table E [TAB] | (PRUNE) bound offsets I [TAB] |
-    // velocity ids [TAB] | list nu float [k * LS] | list vidx u16 [k * LS] | (8-byte aligned)
-    // per-warp queues uint2 [WARPS][QCAP].
+    // velocity ids and entry counts [ROWS] | lists with their buffers: nu float [(k + CAP) * LS],
+    // vidx u16 [(k + CAP) * LS] (KEYS: keys u32 [(k + CAP) * LS]).
     E *s_tab = reinterpret_cast<E *>(s_dyn4);
     I *s_rid = reinterpret_cast<I *>(reinterpret_cast<char *>(s_dyn4) + TAB * EB);
     int *s_vid = reinterpret_cast<int *>(s_rid + (PRUNE ? TAB : 0));
     const int N = a.N, n0 = a.n0, NJ = N - n0, k = a.k;
-    // table row stride: even, so that entries pair into 16-byte loads; compact entries: a
-    // multiple of 4, four to a 16-byte load
-    const int NJP = CE ? (NJ + 3) & ~3 : (NJ + 1) & ~1;
-    int *s_tab4 = reinterpret_cast<int *>(s_dyn4);
-    float *s_ln = reinterpret_cast<float *>(s_vid + TAB);
-    uint16_t *s_lv = reinterpret_cast<uint16_t *>(s_ln + k * LS);
-    uint32_t *s_lk = reinterpret_cast<uint32_t *>(s_vid + TAB);   // KEYS: the lists instead
-    constexpr size_t kSlotBytes = KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t);
-    uint2 *s_q = reinterpret_cast<uint2 *>(s_dyn4) +
-                 ((TAB * (EB + sizeof(int) + (PRUNE ? sizeof(I) : 0)) + (size_t)k * LS * kSlotBytes + 7) / 8);
-
+    const int NJP = (NJ + 3) & ~3;   // table row stride: whole groups of four entries
+    float *s_ln = reinterpret_cast<float *>(s_vid + ROWS);
+    uint16_t *s_lv = reinterpret_cast<uint16_t *>(s_ln + (k + CAP) * LS);
+    uint32_t *s_lk = reinterpret_cast<uint32_t *>(s_vid + ROWS);   // KEYS: the lists instead
     for (int j = threadIdx.x; j < N; j += THREADS)
         s_scale[j] = (STORAGE == KB_F32) ? make_float2(1.0f, 1.0f) : exp_scale(scale_exp(a.scales[a.epoch_of[j]]));
     for (int i = threadIdx.x; i < k * LS; i += THREADS) {
@@ -456,26 +487,26 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     const bool active = y < a.H;
     const T *planes = reinterpret_cast<const T *>(a.planes);
     // element index of this lane's first pixel within a plane (even for 16-bit storage)
-    const I tb = (I)(a.origin + (long long)y * a.pitch + xw + lane * G::PIX);
-    // per-thread base: an entry's loads start at planes_t + idx; zidx instead lands on
-    // this lane's pixels among the zero columns left of row 0 of plane 0 (kSpan >= the
-    // 128 elements a lane reads there)
-    const T *planes_t = planes + tb;
-    const I zidx = (I)(lane * G::PIX) - tb;
-    const unsigned wbit = 1u << warp;
-    uint2 *q = s_q + warp * QCAP;
-    int qn = 0;                       // pending candidates of this warp (warp-uniform)
+    const long long tb = a.origin + (long long)y * a.pitch + xw + lane * G::PIX;
+    typedef LaneBase<T, byte_offsets<STORAGE, KM, KEYS, I>()> LB;
+    const LB lane0(planes, tb);
     const unsigned lt_mask = (1u << lane) - 1u;
 
     float thn[PX];
     int thv[PX];
     uint32_t thk[PX];   // KEYS: the thresholds as keys
+    int off[PX];        // the next free buffer slot of the lane's columns, as an offset from slot 0
+    const int off_lim = (k + CAP) * LS;
 #pragma unroll
     for (int p = 0; p < PX; ++p) {
         thn[p] = -INFINITY;
         thv[p] = kNoV;
         thk[p] = 0u;
+        off[p] = k * LS;
     }
+    float *ln0 = s_ln + threadIdx.x;      // slot 0 of the lane's first column; column p is p * THREADS further
+    uint16_t *lv0 = s_lv + threadIdx.x;
+    uint32_t *lk0 = s_lk + threadIdx.x;
     __syncthreads();
 
     // epochs at the reference time: offset 0 for every velocity (pixels past W read the zero columns)
@@ -491,10 +522,27 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
         }
     }
 
+    // every lane's buffers into its lists
+    auto merge_lists = [&]() {
+#pragma unroll
+        for (int p = 0; p < PX; ++p) {
+            const int n = (off[p] - k * LS) / LS;
+            if constexpr (KEYS)
+                merge_keys<KM, CAP, LS>(lk0 + p * THREADS, k, n, thk[p]);
+            else if constexpr (KM > kKeyMax)
+                insert_values<LS>(ln0 + p * THREADS, lv0 + p * THREADS, k, n, thn[p], thv[p]);
+            else
+                merge_values<KM, CAP, LS>(ln0 + p * THREADS, lv0 + p * THREADS, k, n, thn[p], thv[p]);
+            off[p] = k * LS;
+        }
+    };
+
     // PRUNE: a bound row holds one value per 32 columns, (W + 31) / 32 + SPAN / 32 of them,
     // the value for a span starting at column x at (x >> 5) + SPAN / 32; the reference
-    // epochs' share is fixed
+    // epochs' share is fixed.  A warp whose row lies outside the image (its loads read zeros)
+    // may add any value of the planes: none is negative, so the sum stays a bound.
     const long long RW = (long long)(a.W + 31) / 32 + SPAN / 32;
+    const long long RE = (long long)N * a.H * RW;
     float b0 = 0.0f;
     if constexpr (PRUNE) {
         if (active)
@@ -502,40 +550,47 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
                 b0 = __fadd_ru(b0, __ldg(a.snr2 + ((long long)a.epoch_of[j] * a.H + y) * RW + (xw >> 5) + SPAN / 32));
     }
 
-    const int vchunk = min(a.V, TAB / max(NJP, 1));
+    // Table build: a group of GL lanes takes one velocity, lane by lane its epochs, and keeps
+    // (in time order) those whose shifted band overlaps the image for this CTA.  Leaving the
+    // others out, which had read zero rows from L1, took 10 % of the loads at 12 x 4096^2
+    // (28 % at 2048^2, more on smaller images).
+    const int GL = NJ <= 4 ? 4 : NJ <= 8 ? 8 : NJ <= 16 ? 16 : 32;
+    const int gl = lane & (GL - 1), gs = lane & ~(GL - 1);
+    const unsigned gmask = (GL == 32 ? 0xffffffffu : (1u << GL) - 1u) << gs;
+    const int vchunk = min(a.V, min(ROWS, TAB / max(NJP, 1)));
     for (int c0 = 0; c0 < a.V; c0 += vchunk) {
         const int nc = min(vchunk, a.V - c0);
         __syncthreads();
-        for (int i = threadIdx.x; i < nc; i += THREADS) s_vid[i] = a.vorder[c0 + i];
-        for (int i = threadIdx.x; i < nc * NJ; i += THREADS) {
-            const int vi = i / NJ, jj = i - vi * NJ;   // entry (vi, jj) at vi * NJP + jj
-            const int j = n0 + jj;
-            const int ep = a.epoch_of[j];
-            const int2 o = a.offs[(long long)a.vorder[c0 + vi] * N + j];
-            const int ox = max(-32767, min(32767, o.x)), oy = max(-32767, min(32767, o.y));
-            int mask = 0;
-            if (xw + ox + SPAN > 0 && xw + ox < a.W) {   // the span overlaps the image's columns
-#pragma unroll
-                for (int w = 0; w < WARPS; ++w)
-                    if ((unsigned)(y0 + w + oy) < (unsigned)a.H) mask |= 1 << w;
+        for (int b = warp * (32 / GL); b < nc; b += WARPS * (32 / GL)) {
+            const int vi = b + gs / GL;
+            const bool ok = vi < nc;
+            int cnt = 0;
+            for (int j0 = 0; j0 < NJ; j0 += GL) {
+                const int jj = j0 + gl, j = n0 + jj;
+                int ep = 0, ox = 0, oy = 0;
+                bool keep = false;
+                if (ok && jj < NJ) {
+                    ep = a.epoch_of[j];
+                    const uint32_t o = a.ptab[(long long)(c0 + vi) * NJ + jj];   // packed (dx, dy)
+                    ox = (int)(short)(o & 0xffffu);
+                    oy = (int)o >> 16;
+                    keep = xw + ox + SPAN > 0 && xw + ox < a.W && y0 + oy + WARPS > 0 && y0 + oy < a.H;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, keep) & gmask;
+                const int at = vi * NJP + cnt + __popc(m & lt_mask);
+                if (keep && debug_in(at, TAB, 5)) {
+                    long long g = (long long)ep * a.plane_elems + (long long)oy * a.pitch + ox;
+                    if (STORAGE != KB_F32 && (ox & 1)) g += a.phase1 - 1;   // odd shift: the phase-1 copy
+                    E e;
+                    e.idx = (I)LB::offset(g);
+                    if constexpr (STORAGE != KB_F32) e.sc = sc_of(s_scale[j]);
+                    s_tab[at] = e;
+                    if constexpr (PRUNE)   // the CTA's first row; a warp adds warp * RW
+                        s_rid[at] = (I)(((long long)ep * a.H + y0 + oy) * RW + ((xw + ox) >> 5) + SPAN / 32);
+                }
+                cnt += __popc(m);
             }
-            long long g = (long long)ep * a.plane_elems + (long long)oy * a.pitch + ox;
-            if (STORAGE != KB_F32 && (ox & 1)) g += a.phase1 - 1;   // odd shift: the phase-1 copy
-            if constexpr (CE) {
-                // a warp's loads start at its lane base plus the offset; rows 0..WARPS-1 of the
-                // allocation are zero (the pad rows above plane 0), one per warp
-                const long long zero_rows = -(a.origin + (long long)y0 * a.pitch + xw);
-                if (debug_in(vi * NJP + jj, TAB, 5)) s_tab4[vi * NJP + jj] = (int)(mask ? g : zero_rows);
-            } else {
-                E e;
-                e.idx = (I)g;
-                e.info = mask;
-                if constexpr (STORAGE != KB_F32) e.sc = sc_of(exp_scale(scale_exp(a.scales[ep])));
-                if (debug_in(vi * NJP + jj, TAB, 5)) s_tab[vi * NJP + jj] = e;
-            }
-            if constexpr (PRUNE)   // the CTA's first row; a warp adds warp * RW
-                s_rid[vi * NJP + jj] = mask ? (I)(((long long)ep * a.H + y0 + oy) * RW + ((xw + ox) >> 5) + SPAN / 32)
-                                            : (I)0;
+            if (ok && gl == 0) s_vid[vi] = a.vorder[c0 + vi] | (cnt << 16);
         }
         __syncthreads();
         if (!active) continue;
@@ -547,11 +602,13 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
                     const int mine = vi + lane;
                     float b = b0;
                     if (mine < nc) {
-                        const E *t = s_tab + mine * NJP;
                         const I *rid = s_rid + mine * NJP;
+                        const int n = s_vid[mine] >> 16;
 #pragma unroll 4
-                        for (int jj = 0; jj < NJ; ++jj)
-                            if (t[jj].info & wbit) b = __fadd_ru(b, __ldg(a.snr2 + rid[jj] + (long long)warp * RW));
+                        for (int jj = 0; jj < n; ++jj) {
+                            const long long r = rid[jj] + (long long)warp * RW;
+                            b = __fadd_ru(b, __ldg(a.snr2 + max(0LL, min(RE - 1, r))));
+                        }
                     }
                     todo = __ballot_sync(0xffffffffu, mine < nc && !(__fmul_ru(b, 1.0f + 0x1p-14f) < a.nu_min2_slack));
                 }
@@ -562,191 +619,50 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
                 }
                 vi += __ffs(rest) - 1;
             }
-            const int v = s_vid[vi];
+            const int v = s_vid[vi] & 0xffff, nj = s_vid[vi] >> 16;
             const E *tab = s_tab + vi * NJP;
             float2 acc[PX];
 #pragma unroll
             for (int p = 0; p < PX; ++p) acc[p] = acc0[p];
-            if constexpr (CE && !LONG) {
-                // epochs in batches of C loads in flight (offsets four to a shared load), then
-                // one at a time
-                const int *tab4 = s_tab4 + vi * NJP;
-                int jj = 0;
-                for (; jj + C <= NJ; jj += C) {
-                    LT val[C][P];
-#pragma unroll
-                    for (int q4 = 0; q4 < C; q4 += 4) {
-                        const int4 o = *reinterpret_cast<const int4 *>(tab4 + jj + q4);
-                        const int oo[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const LT *src = reinterpret_cast<const LT *>(planes_t + oo[h]);
-#pragma unroll
-                            for (int p = 0; p < P; ++p) val[q4 + h][p] = gather(src + 32 * p, planes, a.planes_elems, 2);
-                        }
-                    }
-#pragma unroll
-                    for (int q2 = 0; q2 < C; ++q2) {
-#pragma unroll
-                        for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[q2][p], 0u);
-                    }
-                }
-                for (; jj < NJ; ++jj) {
-                    const LT *src = reinterpret_cast<const LT *>(planes_t + tab4[jj]);
-                    LT val[P];
-#pragma unroll
-                    for (int p = 0; p < P; ++p) val[p] = gather(src + 32 * p, planes, a.planes_elems, 3);
-#pragma unroll
-                    for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[p], 0u);
-                }
-            } else if constexpr (CE) {
-                // LONG: every batch of C predicated (warp-uniform), the row padding read but unused
-                const int *tab4 = s_tab4 + vi * NJP;
-                for (int jj = 0; jj < NJ; jj += C) {
-                    LT val[C][P];
-#pragma unroll
-                    for (int q4 = 0; q4 < C; q4 += 4) {
-                        if (jj + q4 < NJ) {
-                            const int4 o = *reinterpret_cast<const int4 *>(tab4 + jj + q4);
-                            const int oo[4] = {o.x, o.y, o.z, o.w};
-#pragma unroll
-                            for (int h = 0; h < 4; ++h) {
-                                if (jj + q4 + h < NJ) {
-                                    const LT *src = reinterpret_cast<const LT *>(planes_t + oo[h]);
-#pragma unroll
-                                    for (int p = 0; p < P; ++p)
-                                        val[q4 + h][p] = gather(src + 32 * p, planes, a.planes_elems, 4);
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int q2 = 0; q2 < C; ++q2) {
-                        if (jj + q2 < NJ) {
-#pragma unroll
-                            for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[q2][p], 0u);
-                        }
-                    }
-                }
-            } else if constexpr (!LONG) {
-                // epochs in batches of C loads in flight, then one at a time
-                int jj = 0;
-                for (; jj + C <= NJ; jj += C) {
-                    LT val[C][P];
-                    uint32_t sx[C];
-#pragma unroll
-                    for (int q2 = 0; q2 < C; q2 += 2) {
-                        E t[2];
-                        if constexpr (STORAGE == KB_F32) {
-                            load_pair(tab + jj + q2, t[0], t[1]);   // one 16-byte shared load
-                        } else {
-                            t[0] = tab[jj + q2];
-                            t[1] = tab[jj + q2 + 1];
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            sx[q2 + h] = entry_sc(t[h]);
-                            const LT *src = reinterpret_cast<const LT *>(planes_t + ((t[h].info & wbit) ? t[h].idx : zidx));
-#pragma unroll
-                            for (int p = 0; p < P; ++p) val[q2 + h][p] = gather(src + 32 * p, planes, a.planes_elems, 2);
-                        }
-                    }
-#pragma unroll
-                    for (int q2 = 0; q2 < C; ++q2) {
-#pragma unroll
-                        for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[q2][p], sx[q2]);
-                    }
-                }
-                for (; jj < NJ; ++jj) {
-                    const E t = tab[jj];
-                    const LT *src = reinterpret_cast<const LT *>(planes_t + ((t.info & wbit) ? t.idx : zidx));
-                    LT val[P];
-#pragma unroll
-                    for (int p = 0; p < P; ++p) val[p] = gather(src + 32 * p, planes, a.planes_elems, 3);
-                    const uint32_t sc = entry_sc(t);
-#pragma unroll
-                    for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[p], sc);
-                }
-            } else {
-                // every batch of C predicated (warp-uniform): the remainder costs one
-                // round trip instead of one per epoch, for more registers
-                for (int jj = 0; jj < NJ; jj += C) {
-                    LT val[C][P];
-                    uint32_t sx[C];
-#pragma unroll
-                    for (int q2 = 0; q2 < C; q2 += 2) {
-                        if (jj + q2 < NJ) {
-                            E t[2];
-                            load_pair(tab + jj + q2, t[0], t[1]);   // the second may be row padding
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                if (jj + q2 + h < NJ) {
-                                    sx[q2 + h] = entry_sc(t[h]);
-                                    const LT *src = reinterpret_cast<const LT *>(
-                                        planes_t + ((t[h].info & wbit) ? t[h].idx : zidx));
-#pragma unroll
-                                    for (int p = 0; p < P; ++p)
-                                        val[q2 + h][p] = gather(src + 32 * p, planes, a.planes_elems, 4);
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int q2 = 0; q2 < C; ++q2) {
-                        if (jj + q2 < NJ) {
-#pragma unroll
-                            for (int p = 0; p < P; ++p) G::acc(acc + p * G::PIX, val[q2][p], sx[q2]);
-                        }
-                    }
+            // the kept epochs in batches of C loads in flight, then one of four, then the
+            // last one to three together (their loads issued before the first sum)
+            int jj = 0;
+            for (; jj + C <= nj; jj += C) add_epochs<STORAGE, P, C>(tab + jj, lane0, planes, a.planes_elems, acc);
+            if constexpr (C > 4) {
+                if (jj + 4 <= nj) {
+                    add_epochs<STORAGE, P, 4>(tab + jj, lane0, planes, a.planes_elems, acc);
+                    jj += 4;
                 }
             }
-            // scoring, then this velocity's candidates appended to the warp's queue; the
-            // lists are updated when 32 or more are pending (the register thresholds stay
-            // conservative meanwhile: a stale threshold only admits more candidates)
-            float nu[PX];
-            uint32_t key[PX];
-            bool cand[PX];
-            bool any = false;
+            if (jj < nj) add_tail<STORAGE, P>(tab + jj, nj - jj, lane0, planes, a.planes_elems, acc);
+            // scoring; candidates go to their pixels' buffers (the thresholds stay conservative
+            // between merges: a stale one only admits more)
+            bool full = false;
 #pragma unroll
             for (int p = 0; p < PX; ++p) {
                 const float F = acc[p].y;
-                nu[p] = acc[p].x * rsqrtf(F);
+                const float nu = acc[p].x * rsqrtf(F);
                 if constexpr (KEYS) {
-                    key[p] = nu_key(nu[p], v, a.key_bits);
-                    cand[p] = (F > 0.0f) && (nu[p] >= a.nu_min) && key[p] > thk[p];
+                    const uint32_t key = nu_key(nu, v, a.key_bits);
+                    if ((F > 0.0f) && (nu >= a.nu_min) && key > thk[p] && debug_in(off[p], off_lim, 6)) {
+                        lk0[p * THREADS + off[p]] = key;
+                        off[p] += LS;
+                        full |= off[p] == off_lim;
+                    }
                 } else {
-                    key[p] = __float_as_uint(nu[p]);
-                    cand[p] = (F > 0.0f) && (nu[p] >= a.nu_min) && better(nu[p], v, thn[p], thv[p]);
+                    if ((F > 0.0f) && (nu >= a.nu_min) && better(nu, v, thn[p], thv[p]) && debug_in(off[p], off_lim, 6)) {
+                        ln0[p * THREADS + off[p]] = nu;
+                        lv0[p * THREADS + off[p]] = (uint16_t)v;
+                        off[p] += LS;
+                        full |= off[p] == off_lim;
+                    }
                 }
-                any |= cand[p];
             }
-            if (!__any_sync(0xffffffffu, any)) continue;
-#pragma unroll
-            for (int p = 0; p < PX; ++p) {
-                const unsigned m = __ballot_sync(0xffffffffu, cand[p]);
-                if (cand[p])
-                    q[qn + __popc(m & lt_mask)] = make_uint2(key[p], (unsigned)v | ((unsigned)(p * 32 + lane) << 16));
-                qn += __popc(m);
-            }
-            if (qn >= 32) {
-                __syncwarp();
-                if constexpr (KEYS)
-                    flush_keys<PX>(q, qn, s_lk, k, LS, warp, lane, thk);
-                else
-                    flush_queue<PX, LONG>(q, qn, s_ln, s_lv, k, LS, warp, lane, thn, thv);
-                qn = 0;
-            }
+            if (__any_sync(0xffffffffu, full)) merge_lists();
         }
     }
     if (!active) return;
-    if (qn > 0) {
-        __syncwarp();
-        if constexpr (KEYS)
-            flush_keys<PX>(q, qn, s_lk, k, LS, warp, lane, thk);
-        else
-            flush_queue<PX, LONG>(q, qn, s_ln, s_lv, k, LS, warp, lane, thn, thv);
-    }
-    __syncwarp();
+    merge_lists();
     if constexpr (KEYS) {
         // candidates for the rescoring, best first, as the keys themselves (4 bytes each,
         // decoded by the rescoring, which recomputes the sums)
@@ -826,22 +742,20 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     }
 }
 
-// Resident CTAs per SM the register allocation is held to (0: no hold), by
-// shape.  Lists up to 8 long (plain remainder loop): the narrow shapes (FP32 with
-// two pixels per lane, 16-bit with one pixel pair) are held to 5 CTAs (48
-// registers; shared memory allows 5 at k = 8); 16-bit with two pixel pairs per
-// lane to 3 with 4-epoch batches (80 registers; the k = 8 lists of its 1024-pixel
-// CTAs allow 3) and 2 with 8-epoch batches.  Longer lists (predicated remainder,
-// shared memory for 2-3 CTAs): 3.  The wide FP32 shapes: 2.  The batch kernel,
-// which keeps its search's arguments in shared memory rather than the parameter
-// bank and so needs more registers, is held to 3 for the narrow shapes and 2 for
-// the others.
-template <int STORAGE, int P, int C, bool LONG>
+// Resident CTAs per SM the register allocation is held to, by shape.  Lists up to 8
+// long: the narrow shapes (FP32 with two pixels per lane, 16-bit with one pixel pair) are
+// held to 4 CTAs (64 registers: the loop keeps everything in registers; at 5 CTAs, 48
+// registers, it spills in the loop: 12 x 4096^2, k = 8, 136 ms against 76); 16-bit with
+// two pixel pairs per lane to 3 with 4-epoch batches (80 registers) and 2 with 8-epoch
+// batches.  Longer lists: 3.  The wide FP32 shapes: 2.  The batch kernel, which keeps its
+// search's arguments in shared memory rather than the parameter bank and so needs more
+// registers, is held to 3 for the narrow shapes and 2 for the others.
+template <int STORAGE, int P, int C, int KM, bool KEYS>
 constexpr int min_ctas() {
     constexpr bool narrow = STORAGE == KB_F32 ? P <= 2 : P <= 1;
-    if (STORAGE != KB_F32 && P == 2) return (C <= 4 && !LONG) ? 3 : 2;
+    if (STORAGE != KB_F32 && P == 2) return (C <= 4 && KM <= kKeyMax && (KEYS || KM <= kShortMax)) ? 3 : 2;
     if (!narrow) return 2;
-    return LONG ? 3 : 5;
+    return KM > kShortMax ? 3 : 4;
 }
 
 template <int STORAGE, int P>
@@ -849,8 +763,8 @@ constexpr int min_ctas_batch() {
     return (STORAGE == KB_F32 ? P <= 2 : P <= 1) ? 3 : 2;
 }
 
-template <int STORAGE, int P, int C, bool LONG, typename I, bool PRUNE, bool KEYS>
-__global__ void __launch_bounds__(THREADS, (PRUNE && min_ctas<STORAGE, P, C, LONG>() == 5) ? 4 : min_ctas<STORAGE, P, C, LONG>())
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS>
+__global__ void __launch_bounds__(THREADS, min_ctas<STORAGE, P, C, KM, KEYS>())
     search_kernel(SearchArgs a) {
     __shared__ float2 s_scale[KB_MAX_EPOCHS];
     extern __shared__ int4 s_dyn4[];
@@ -864,14 +778,14 @@ __global__ void __launch_bounds__(THREADS, (PRUNE && min_ctas<STORAGE, P, C, LON
         by = r / w;
         bx = s * a.swz + (r - by * w);
     }
-    search_tile<STORAGE, P, C, LONG, I, PRUNE, KEYS>(a, bx, a.by0 + by, s_scale, s_dyn4);
+    search_tile<STORAGE, P, C, KM, I, PRUNE, KEYS>(a, bx, a.by0 + by, s_scale, s_dyn4);
 }
 
 // Persistent batch search: CTAs take (job, tile) work items from an atomic
 // counter until the list is exhausted, copying the item's job descriptor into
 // shared memory first.  The item list is ordered by cost (largest first), so
 // uneven stacks, grids and epoch counts balance across the SMs.
-template <int STORAGE, int P, int C, bool LONG, typename I>
+template <int STORAGE, int P, int C, int KM, typename I>
 __global__ void __launch_bounds__(THREADS, min_ctas_batch<STORAGE, P>())
     search_batch_kernel(const SearchArgs *jobs, const int4 *items, int n_items, int *counter) {
     __shared__ float2 s_scale[KB_MAX_EPOCHS];
@@ -887,28 +801,28 @@ __global__ void __launch_bounds__(THREADS, min_ctas_batch<STORAGE, P>())
         for (int i = threadIdx.x; i < (int)(sizeof(SearchArgs) / sizeof(int)); i += THREADS)
             reinterpret_cast<int *>(&s_job)[i] = reinterpret_cast<const int *>(jobs + w.x)[i];
         __syncthreads();
-        search_tile<STORAGE, P, C, LONG, I, false>(s_job, w.y, w.z, s_scale, s_dyn4);
+        search_tile<STORAGE, P, C, KM, I, false>(s_job, w.y, w.z, s_scale, s_dyn4);
         __syncthreads();
     }
 }
 
-// dynamic shared memory of a CTA with lists of k entries: the table, the lists and the queues
-template <int STORAGE, int P, typename I, bool PRUNE = false, bool KEYS = false>
+// dynamic shared memory of a CTA with lists of k entries: the table, and the lists with their buffers
+template <int STORAGE, int P, int KM, typename I, bool PRUNE = false, bool KEYS = false>
 size_t tile_smem(int k) {
     constexpr int PX = P * Gather<STORAGE>::PIX;
-    const size_t base = (size_t)table_entries<STORAGE, I, PRUNE>() *
-                            (table_entry_bytes<STORAGE, I, PRUNE>() + sizeof(int) + (PRUNE ? sizeof(I) : 0)) +
-                        (size_t)k * THREADS * PX * (KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t));
-    return (base + 7) / 8 * 8 + (size_t)WARPS * 32 * (PX + 1) * sizeof(uint2);
+    constexpr int TAB = table_entries<STORAGE, I, PRUNE>();
+    return (size_t)TAB * (table_entry_bytes<STORAGE, I>() + (PRUNE ? sizeof(I) : 0)) + TAB / 4 * sizeof(int) +
+           (size_t)(k + list_cap<KM, KEYS, PX>()) * THREADS * PX *
+               (KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t));
 }
 
-template <int STORAGE, int P, int C, bool LONG, typename I, bool PRUNE, bool KEYS = false>
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false>
 cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
     constexpr int SPAN = 32 * P * Gather<STORAGE>::PIX;
     static_assert(SPAN <= kSpan, "warp span wider than the zero columns");
-    auto kern = search_kernel<STORAGE, P, C, LONG, I, PRUNE, KEYS>;
+    auto kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS>;
     dim3 grid((a.W + SPAN - 1) / SPAN, a.nby > 0 ? a.nby : (a.H + WARPS - 1) / WARPS);
-    const size_t smem = tile_smem<STORAGE, P, I, PRUNE, KEYS>(a.k);
+    const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // Shared-memory carveout: the driver's choice unless the caller sets one
     // (kb_set_search_carveout); it trades resident CTAs against the L1 that the
@@ -920,19 +834,19 @@ cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// lists longer than kRankMax take the walking insertion and the predicated remainder
+// the merge by the lists' length (candidate lists reach 24: k = 16, BF16)
 template <int STORAGE, int P, int C, typename I, bool PRUNE>
 cudaError_t launch_one(const SearchArgs &a, cudaStream_t st) {
-    if (a.k > kRankMax) return launch_pt<STORAGE, P, C, true, I, PRUNE>(a, st);
-    return launch_pt<STORAGE, P, C, false, I, PRUNE>(a, st);
+    if (a.k > kKeyMax) return launch_pt<STORAGE, P, C, kListMax, I, PRUNE>(a, st);
+    if (a.k > kShortMax) return launch_pt<STORAGE, P, C, kKeyMax, I, PRUNE>(a, st);
+    return launch_pt<STORAGE, P, C, kShortMax, I, PRUNE>(a, st);
 }
 
 // the candidate search of the FP64 rescoring in key form (automatic shape, no pruning)
 template <int STORAGE, int P, int C>
 cudaError_t launch_keys(const SearchArgs &a, cudaStream_t st) {
-    const long long span = (STORAGE == KB_F32 ? 1LL : 2LL) * a.N * a.plane_elems;
-    if (span < (1LL << 31) - 1) return launch_pt<STORAGE, P, C, false, int, false, true>(a, st);
-    return launch_pt<STORAGE, P, C, false, long long, false, true>(a, st);
+    if (search_idx32(a)) return launch_pt<STORAGE, P, C, kKeyMax, int, false, true>(a, st);
+    return launch_pt<STORAGE, P, C, kKeyMax, long long, false, true>(a, st);
 }
 
 // key form where it keeps at least 11 of nu's 23 fraction bits (up to 4096 velocities)
@@ -940,19 +854,18 @@ bool use_keys(const SearchArgs &a) {
     return a.cand_only && !a.snr2 && a.k <= kKeyMax && a.key_bits >= 1 && a.key_bits <= 12;
 }
 
-// 32-bit element offsets when every plane of both phases (and the bound planes) fits
+// 32-bit offsets when every plane of both phases (and the bound planes) fits
 template <int STORAGE, int P, int C, bool PRUNE = false>
 cudaError_t launch_idx(const SearchArgs &a, cudaStream_t st) {
-    const long long span = (STORAGE == KB_F32 ? 1LL : 2LL) * a.N * a.plane_elems;
     const long long rspan = PRUNE ? (long long)a.N * a.H * ((a.W + 31) / 32 + P * Gather<STORAGE>::PIX) : 0;
-    if (span < (1LL << 31) - 1 && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
+    if (search_idx32(a) && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
     return launch_one<STORAGE, P, C, long long, PRUNE>(a, st);
 }
 
 // Shapes: (loads per lane P, epochs per load batch C); a 16-bit load is two pixels.
-// Defaults (variant 0), measured on the 12 x 4096^2 stack at k = 8: FP32 (2, 8)
-// 88 ms against 89 for (2, 4); 16-bit (2, 4): BF16 80 ms against 91 for (1, 4),
-// 96 for (2, 8) and 112 for (1, 8).
+// Defaults (variant 0): FP32 (2, 8), 12 x 4096^2, k = 8: 76 ms; 16-bit value lists (1, 8),
+// 1500 x 1700, 10 epochs, 500 velocities, BF16 / FP16 at k = 8: 6.32 / 6.26 ms, (1, 4) 6.87 /
+// 6.15, (2, 8) 7.29 / 7.19, (2, 4) 7.52 / 7.49; BF16 at k = 12: 8.40, (1, 4) 9.50, (2, 8) 11.1.
 template <int STORAGE>
 cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
     if constexpr (STORAGE == KB_F32) {
@@ -971,22 +884,23 @@ cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
             case 3: return launch_idx<STORAGE, 2, 8>(a, st);
             case 4: return launch_idx<STORAGE, 1, 8>(a, st);
             case 1: return launch_idx<STORAGE, 2, 4>(a, st);
-            // automatic: lists longer than kRankMax take the one-pair shape, whose 512-pixel
-            // CTAs keep their lists' shared memory within what 3 CTAs per SM can hold
+            // automatic: key lists take two pairs per lane; value lists one pair, whose merges
+            // fit the registers beside the loop (and pruned short ones two, as their bound
+            // planes' span has it)
             default:
                 if (use_keys(a)) return launch_keys<STORAGE, 2, 4>(a, st);
                 if (a.snr2)
-                    return a.k > kRankMax ? launch_idx<STORAGE, 1, 4, true>(a, st) : launch_idx<STORAGE, 2, 4, true>(a, st);
-                return a.k > kRankMax ? launch_idx<STORAGE, 1, 4>(a, st) : launch_idx<STORAGE, 2, 4>(a, st);
+                    return a.k > kShortMax ? launch_idx<STORAGE, 1, 4, true>(a, st) : launch_idx<STORAGE, 2, 4, true>(a, st);
+                return launch_idx<STORAGE, 1, 8>(a, st);
         }
     }
 }
 
-template <int STORAGE, int P, int C, bool LONG, typename I>
+template <int STORAGE, int P, int C, int KM, typename I>
 cudaError_t launch_batch_pt(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int kmax,
                             int carve, int sm_count, cudaStream_t st) {
-    const size_t smem = tile_smem<STORAGE, P, I>(kmax);
-    auto kern = search_batch_kernel<STORAGE, P, C, LONG, I>;
+    const size_t smem = tile_smem<STORAGE, P, KM, I>(kmax);
+    auto kern = search_batch_kernel<STORAGE, P, C, KM, I>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err == cudaSuccess && carve >= 0)
         err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
@@ -1002,9 +916,11 @@ cudaError_t launch_batch_pt(const SearchArgs *jobs, const int4 *items, int n_ite
 template <int STORAGE, int P, int C, typename I>
 cudaError_t launch_batch_one(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int kmax,
                              int carve, int sm_count, cudaStream_t st) {
-    if (kmax > kRankMax)
-        return launch_batch_pt<STORAGE, P, C, true, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
-    return launch_batch_pt<STORAGE, P, C, false, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+    if (kmax > kKeyMax)
+        return launch_batch_pt<STORAGE, P, C, kListMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+    if (kmax > kShortMax)
+        return launch_batch_pt<STORAGE, P, C, kKeyMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+    return launch_batch_pt<STORAGE, P, C, kShortMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
 }
 
 template <int STORAGE, int P, int C>
@@ -1037,27 +953,62 @@ cudaError_t launch_batch_storage(const SearchArgs *jobs, const int4 *items, int 
 
 }  // namespace
 
+template <>
+cudaError_t launch_search_storage<KB_SEARCH_STORAGE>(const SearchArgs &a, cudaStream_t st) {
+    return launch_storage<KB_SEARCH_STORAGE>(a, st);
+}
+template <>
+cudaError_t launch_search_batch_storage<KB_SEARCH_STORAGE>(const SearchArgs *jobs, const int4 *items, int n_items,
+                                                           int *counter, int variant, int kmax, int carve, bool idx64,
+                                                           int sm_count, cudaStream_t st) {
+    return launch_batch_storage<KB_SEARCH_STORAGE>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+}
+template <>
+cudaError_t debug_word_storage<KB_SEARCH_STORAGE>(unsigned long long *word, bool reset) {
+#ifdef KB_DEBUG
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpyFromSymbol(word, g_debug_word, sizeof(*word));
+    if (e == cudaSuccess && reset) {
+        const unsigned long long zero = 0;
+        e = cudaMemcpyToSymbol(g_debug_word, &zero, sizeof(zero));
+    }
+    return e;
+#else
+    (void)word;
+    (void)reset;
+    return cudaErrorNotSupported;
+#endif
+}
+
+#ifdef KB_SEARCH_COMMON
+
+cudaError_t debug_word(unsigned long long *word, bool reset) {
+    unsigned long long w[3] = {0, 0, 0};
+    cudaError_t e = debug_word_storage<KB_F32>(&w[0], reset);
+    if (e == cudaSuccess) e = debug_word_storage<KB_BF16>(&w[1], reset);
+    if (e == cudaSuccess) e = debug_word_storage<KB_F16>(&w[2], reset);
+    *word = w[0] ? w[0] : w[1] ? w[1] : w[2];
+    return e;
+}
+
 int search_span(int storage, int variant, int k) {
     // loads per lane P of the shape, times 32 lanes, times pixels per load
     static const int p32[5] = {2, 4, 2, 4, 2}, p16[5] = {2, 2, 1, 2, 1};
     const int v = (variant >= 1 && variant <= 4) ? variant : 0;
-    if (storage != KB_F32 && v == 0 && k > kRankMax) return 64;
+    if (storage != KB_F32 && v == 0 && k > kShortMax) return 64;
     return storage == KB_F32 ? 32 * p32[v] : 64 * p16[v];
 }
 
-int search_auto_span(int storage, int k) { return search_span(storage, 0, k); }
+int search_auto_span(int storage, int k) { return search_span(storage, 0, k); }   // of the pruned search
 
-int default_variant(int storage, int k) {
-    if (storage == KB_F32) return 4;       // (2, 8)
-    return k > kRankMax ? 2 : 1;           // (1, 4) / (2, 4)
-}
+int default_variant(int, int) { return 4; }   // (2, 8), 16-bit (1, 8)
 
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
                                 int variant, int kmax, int carve, bool idx64, int sm_count, cudaStream_t st) {
     switch (storage) {
-        case KB_F32: return launch_batch_storage<KB_F32>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
-        case KB_BF16: return launch_batch_storage<KB_BF16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
-        case KB_F16: return launch_batch_storage<KB_F16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+        case KB_F32: return launch_search_batch_storage<KB_F32>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+        case KB_BF16: return launch_search_batch_storage<KB_BF16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+        case KB_F16: return launch_search_batch_storage<KB_F16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1066,11 +1017,13 @@ bool search_keys(const SearchArgs &a) { return a.variant == 0 && use_keys(a); }
 
 cudaError_t launch_search(const SearchArgs &a, cudaStream_t st) {
     switch (a.storage) {
-        case KB_F32: return launch_storage<KB_F32>(a, st);
-        case KB_BF16: return launch_storage<KB_BF16>(a, st);
-        case KB_F16: return launch_storage<KB_F16>(a, st);
+        case KB_F32: return launch_search_storage<KB_F32>(a, st);
+        case KB_BF16: return launch_search_storage<KB_BF16>(a, st);
+        case KB_F16: return launch_search_storage<KB_F16>(a, st);
         default: return cudaErrorInvalidValue;
     }
 }
+
+#endif  // KB_SEARCH_COMMON
 
 }  // namespace kb
