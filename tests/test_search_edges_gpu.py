@@ -100,3 +100,43 @@ def test_key_lists_at_their_lengths(kb, ctx, storage, k):
     assert got.tobytes() == ref.tobytes()
     for o in (s, f):
         o.free()
+
+
+@pytest.mark.parametrize("N,H,W,k", [(5, 9, 255, 3), (16, 6, 257, 8), (17, 5, 300, 16), (32, 4, 70, 1), (33, 6, 40, 5),
+                                     (70, 3, 33, 2)])
+def test_filter_against_direct_sums(kb, ctx, N, H, W, k):
+    """Epochs held in registers (up to 16, up to 32) or gathered again, strips of 256 pixels: sums,
+    rejections and scores of the direct FP64 form, which rounds alike step by step."""
+    st = synth.small_stack(200 + N, N, H, W, K=5, nan_frac=0.1, n_angles=6, n_speeds=6, s_hi=12.0, n_sources=3, flux=60.0)
+    s = _stack(kb, ctx, st, "f32")
+    job = kb.Job(ctx, H, W, N, st.vx.size, k)
+    job.search(s, st.times, st.vx, st.vy)
+    rec, got = job.results(), job.filter_lightcurves(s, 2.5)
+    planes = np.empty((N, H, W, 2), np.float32)
+    s.copy_planes(0, planes)
+    dx, dy = kb.offsets(st.times, st.vx, st.vy)
+    y, x, _ = np.meshgrid(np.arange(H), np.arange(W), np.arange(k), indexing="ij")
+    v, order, q = np.maximum(rec["vidx"], 0), np.argsort(st.times, kind="stable"), {}
+    P, F = np.zeros((H, W, k)), np.zeros((H, W, k))
+    for e in order:
+        yy, xx = y + dy[v, e], x + dx[v, e]
+        ok = (rec["vidx"] >= 0) & (yy >= 0) & (yy < H) & (xx >= 0) & (xx < W)
+        q[e] = np.where(ok[..., None], planes[e][np.clip(yy, 0, H - 1), np.clip(xx, 0, W - 1)].astype(np.float64), 0.0), ok
+        P, F = P + q[e][0][..., 0], F + q[e][0][..., 1]
+    Pk, Fk, n, bits = np.zeros_like(P), np.zeros_like(P), np.zeros(P.shape, int), np.zeros(P.shape + (4,), np.uint32)
+    for e in order:
+        (pe, fe), ok = (q[e][0][..., 0], q[e][0][..., 1]), q[e][1]
+        rest = F - fe
+        out = ok & (fe > 0) & (rest > 0) & ((pe * F - P * fe) ** 2 > 6.25 * F * fe * rest)
+        keep = ok & ~out
+        Pk, Fk, n = Pk + np.where(keep, pe, 0.0), Fk + np.where(keep, fe, 0.0), n + keep
+        bits[..., e // 32] |= np.where(out, np.uint32(1 << (e % 32)), np.uint32(0)).astype(np.uint32)
+    assert np.array_equal(got["rejected"], bits) and np.array_equal(got["nobs"], n)
+    assert np.array_equal(got["nrejected"], sum(((bits >> b) & 1).sum(-1) for b in range(32)))
+    assert np.array_equal(got["psi"], Pk) and np.array_equal(got["phi"], Fk)
+    ok = Fk > 0
+    assert np.array_equal(got["nu"][ok], Pk[ok] / np.sqrt(Fk[ok])) and np.all(got["nu"][~ok] == -np.inf)
+    assert np.array_equal(got["alpha"][ok], Pk[ok] / Fk[ok]) and (bits.any() or H * W < 200)
+    assert np.array_equal(got["x0"], x) and np.array_equal(got["y0"], y) and np.array_equal(got["vidx"], rec["vidx"])
+    job.free()
+    s.free()
