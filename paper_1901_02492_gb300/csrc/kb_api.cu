@@ -1542,9 +1542,9 @@ int kb_cluster(kb_ctx *ctx, const kb_result *cand, size_t n, const kb_cluster_pa
     cudaStream_t st = (cudaStream_t)stream;
     int T = 1;
     while (T < 2 * (int)n) T <<= 1;
-    const size_t words = 2 * (size_t)T + 3 * n;   // owner, head | next, parent, bestidx
-    const size_t bytes = 2 * n * sizeof(int4) + n * sizeof(unsigned long long) + words * sizeof(int) +
-                         2 * sizeof(int) + 2 * n + 16;
+    const size_t words = 3 * (size_t)T + 5 * n;   // owner, cnt, start | slot, rank, run_idx, parent, bestidx
+    const size_t bytes = 3 * n * sizeof(int4) + n * sizeof(unsigned long long) + words * sizeof(int) +
+                         3 * sizeof(int) + 2 * n + 16;
     void *buf = nullptr;
     size_t acct = 0;
     int rc = dev_alloc(ctx, bytes, &buf, &acct);
@@ -1559,20 +1559,32 @@ int kb_cluster(kb_ctx *ctx, const kb_result *cand, size_t n, const kb_cluster_pa
     // cells a little wider than eps: the rounding of the weighted coordinates
     // cannot put two neighbours more than one cell apart
     a.inv_side = 1.0 / (p->eps * (1.0 + 1.0 / 1048576.0));
+    // FP32 distances decide away from eps2 (kb_cluster.cu, within()); where they could
+    // overflow or lose accuracy near the subnormal range they decide nothing
+    const bool f32 = a.eps2 > 1e-20 && a.eps2 < 1e20 && a.w_pos > 1e-15 && a.w_pos < 1e15 && a.w_vel > 1e-15 &&
+                     a.w_vel < 1e15 &&
+                     p->eps < p->w_pos * 536870912.0;   // neighbours' pixel differences fit 31 bits
+    a.eps2_lo = f32 ? (float)(a.eps2 * (1.0 - 0x1p-16)) : NAN;
+    a.eps2_hi = f32 ? (float)(a.eps2 * (1.0 + 0x1p-16)) : NAN;
     a.min_samples = p->min_samples;
     a.pts = reinterpret_cast<int4 *>(buf);
     a.cells = a.pts + n;
-    unsigned long long *bestnu = reinterpret_cast<unsigned long long *>(a.cells + n);
+    a.run_pts = a.cells + n;
+    unsigned long long *bestnu = reinterpret_cast<unsigned long long *>(a.run_pts + n);
     int *w = reinterpret_cast<int *>(bestnu + n);
     a.bestnu = bestnu;
     a.owner = w;
-    a.head = w + T;
-    a.next = w + 2 * (size_t)T;
-    a.parent = a.next + n;
+    a.cnt = w + T;
+    a.start = w + 2 * (size_t)T;
+    a.slot = w + 3 * (size_t)T;
+    a.rank = a.slot + n;
+    a.run_idx = a.rank + n;
+    a.parent = a.run_idx + n;
     a.bestidx = a.parent + n;
     a.count = reinterpret_cast<unsigned *>(a.bestidx + n);
     a.status = reinterpret_cast<int *>(a.count + 1);
-    a.core = reinterpret_cast<uint8_t *>(a.status + 1);
+    a.cursor = a.status + 1;
+    a.core = reinterpret_cast<uint8_t *>(a.cursor + 1);
     a.valid = a.core + n;
     a.label = label;
     a.keep = keep;

@@ -366,10 +366,15 @@ struct ClusterArgs {
     int n, T;                // candidates, hash slots (a power of two >= 2n)
     double w_pos, w_vel, eps2, inv_side;
     int min_samples;
+    float eps2_lo, eps2_hi;  // FP32 distances below / above these are decided (NaN: none is)
     int4 *pts, *cells;       // [n] packed (x0, y0, vx bits, vy bits), grid cell
+    int4 *run_pts;           // [n] the points, cell by cell
     uint8_t *valid;          // [n] takes part (vidx >= 0, cell in range)
-    int *owner, *head;       // [T] first candidate of the slot's cell, list head
-    int *next, *parent;      // [n]
+    int *owner, *cnt, *start;  // [T] first candidate of the slot's cell, its points, their run in run_pts
+    int *slot, *rank;        // [n] the point's slot and its place in the run
+    int *run_idx;            // [n] candidate of run_pts
+    int *parent;             // [n]
+    int *cursor;             // places given out
     uint8_t *core;           // [n]
     unsigned long long *bestnu;  // [n] per group: ordered bits of the best nu
     int *bestidx;            // [n] per group: lowest index reaching it

@@ -140,3 +140,36 @@ def test_filter_against_direct_sums(kb, ctx, N, H, W, k):
     assert np.array_equal(got["x0"], x) and np.array_equal(got["y0"], y) and np.array_equal(got["vidx"], rec["vidx"])
     job.free()
     s.free()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 700])
+@pytest.mark.parametrize("eps", [2.0, 5.0])
+def test_cluster_on_a_lattice(kb, ctx, n, eps):
+    """Whole-pixel spacings: many pairs lie at eps exactly, cells hold up to hundreds of points."""
+    rng = np.random.default_rng(n)
+    rec = np.zeros(n, kb.RESULT_DTYPE)
+    rec["x0"], rec["y0"] = rng.integers(0, 24, n), rng.integers(0, 24, n)
+    rec["vx"], rec["vy"] = rng.integers(0, 3, n), rng.integers(0, 3, n)
+    rec["vidx"], rec["nu"] = rng.integers(-1, 40, n), rng.normal(5.0, 2.0, n)
+    dev = torch.from_numpy(rec.view(np.uint8).copy()).to(DEV)
+    for ms in (1, 4, 40):
+        label, keep, core, groups = ctx.cluster(dev, 1.0, 1.0, eps, ms, core=True)
+        p = np.stack([rec["x0"], rec["y0"], rec["vx"], rec["vy"]], 1).astype(np.float64)
+        d2, ok = ((p[:, None] - p[None]) ** 2).sum(-1), rec["vidx"] >= 0   # exact: small whole numbers
+        near = (d2 <= eps * eps) & ok[:, None] & ok[None]
+        want_core = ok & (near.sum(1) >= ms)
+        want = np.where(ok, np.arange(n), -1)
+        link = near & want_core[:, None] & want_core[None]
+        for _ in range(n):
+            low = np.where(link, want[None], n).min(1, initial=n)
+            new = np.where(want_core, np.minimum(want, low), want)
+            if np.array_equal(new, want):
+                break
+            want = new
+        for i in np.flatnonzero(ok & ~want_core):
+            c = np.flatnonzero(near[i] & want_core)
+            if c.size:
+                want[i] = want[c[np.lexsort((c, d2[i, c]))[0]]]
+        assert np.array_equal(label.cpu().numpy(), want)
+        assert np.array_equal(core.cpu().numpy(), want_core)
+        assert groups == np.unique(want[ok]).size == int(keep.sum())
