@@ -590,13 +590,18 @@ cudaError_t launch_gen(const PsiPhiArgs &a, dim3, size_t, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// streaming separable kernel: segments of up to 512 rows (a 2 r-row warm-up each,
-// 3 % of 512 for K = 17), one CTA per (strip, segment, epoch)
+// streaming separable kernel, one CTA per (strip, segment, epoch): segments of up to 512
+// rows (a 2 r-row warm-up each, 3 % of 512 for K = 17), halved down to one batch of rows
+// while the launch would leave places for resident CTAs (3 per SM) empty: 9 x 512 x 512,
+// K = 13, whole columns are 72 CTAs and 47 us, segments of 64 rows 576 CTAs and 25 us;
+// 5 x 64 x 64, K = 7: 8.7 us against 7.6
 template <int KT>
 cudaError_t launch_stream(const PsiPhiArgs &a0, cudaStream_t st) {
     typedef StreamGeom<KT> G;
     PsiPhiArgs a = a0;
     a.seg = std::min(512, (a.H + SY - 1) / SY * SY);
+    const long long strips = (long long)((a.W + TX - 1) / TX) * a.N;
+    while (a.seg > SY && strips * ((a.H + a.seg - 1) / a.seg) < 152 * 3) a.seg = (a.seg / 2 + SY - 1) / SY * SY;
     const dim3 grid((a.W + TX - 1) / TX, (a.H + a.seg - 1) / a.seg, a.N);
     const size_t smem = G::taps_bytes + G::raw_bytes + G::a_bytes + G::ring_bytes + (a.mask ? G::mask_bytes : 0);
     cudaError_t err = cudaFuncSetAttribute(psi_phi_stream_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -173,3 +173,28 @@ def test_cluster_on_a_lattice(kb, ctx, n, eps):
         assert np.array_equal(label.cpu().numpy(), want)
         assert np.array_equal(core.cpu().numpy(), want_core)
         assert groups == np.unique(want[ok]).size == int(keep.sum())
+
+
+@pytest.mark.parametrize("N,H,W,K", [(1, 1, 1, 3), (3, 33, 63, 7), (2, 70, 66, 13), (9, 130, 129, 21), (1, 1200, 64, 5),
+                                     (4, 97, 1027, 17)])
+def test_streaming_images_equal_the_tile_kernel(kb, ctx, N, H, W, K):
+    """Aligned and ragged widths, short and split columns, against the tile kernel: the same PSF within
+    23 x 23 taps, whose added zeros change no sum.  Planes, and the 16-bit codes, copied to both kinds of memory."""
+    st = synth.small_stack(N + K, N, H, W, K=K, nan_frac=0.05, mask_frac=0.05, n_sources=1, flux=50.0)
+    wide = np.zeros((N, 23, 23), np.float32)
+    o = (23 - K) // 2
+    wide[:, o:o + K, o:o + K] = st.psf
+    mask = torch.from_numpy((np.arange(N * H * W).reshape(N, H, W) % 37 == 0).astype(np.uint8)).to(DEV)
+    got = []
+    for psf in (st.psf, wide):
+        s = kb.Stack(ctx, N, H, W, "f16")
+        s.make_psi_phi(torch.from_numpy(st.sci).to(DEV), torch.from_numpy(st.var).to(DEV), mask, psf)
+        for which, dt, kind in ((0, torch.float32, np.float32), (1, torch.int16, np.int16)):
+            d = torch.empty((N, H, W, 2), dtype=dt, device=DEV)
+            h = np.empty((N, H, W, 2), kind)
+            s.copy_planes(which, d)
+            s.copy_planes(which, h)
+            assert np.array_equal(d.cpu().numpy(), h)
+            got.append(h)
+        s.free()
+    assert np.array_equal(got[0], got[2]) and np.array_equal(got[1], got[3])
