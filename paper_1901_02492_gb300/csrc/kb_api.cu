@@ -503,7 +503,14 @@ int kb_stack_copy_planes(const kb_stack *s, int which, void *dst, size_t dst_byt
     cudaStream_t st = (cudaStream_t)stream;
     bool dev = is_device_ptr(dst);
     cudaError_t e = cudaSuccess;
-    for (int ep = 0; ep < s->N && e == cudaSuccess; ++ep) {
+    // one kernel where dst is this device's own memory and its elements are aligned
+    cudaPointerAttributes at;
+    const bool here = dev && (uintptr_t)dst % elem == 0 && cudaPointerGetAttributes(&at, dst) == cudaSuccess &&
+                      at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+    if (here)
+        e = kb::launch_copy_rows((const char *)src + (size_t)s->L.origin * elem, dst, elem, s->N, s->H, s->W, s->L.pitch,
+                                 s->L.plane_elems, st);
+    for (int ep = 0; !here && ep < s->N && e == cudaSuccess; ++ep) {
         const char *from = (const char *)src + (size_t)(ep * s->L.plane_elems + s->L.origin) * elem;
         char *to = (char *)dst + (size_t)ep * s->H * s->W * elem;
         e = cudaMemcpy2DAsync(to, (size_t)s->W * elem, from, (size_t)s->L.pitch * elem, (size_t)s->W * elem,

@@ -186,6 +186,9 @@ struct PsiPhiArgs {
 cudaError_t launch_psi_phi(const PsiPhiArgs &a, cudaStream_t st);
 cudaError_t launch_quantize(const float2 *f32, pair16 *q16, float2 *scales, const unsigned *maxbits, int N,
                             long long plane_elems, int storage, cudaStream_t st);
+// the planes' rows (src at pixel (0, 0) of epoch 0; elem 8 or 4 bytes) into dst [N][H][W] on the same device
+cudaError_t launch_copy_rows(const void *src, void *dst, size_t elem, int N, int H, int W, int pitch,
+                             long long plane_elems, cudaStream_t st);
 // layout helper: floats needed for the taps of N epochs with kernel size K
 size_t taps_floats(int N, int K, bool separable);
 // rank-1 test and factors of a K x K PSF, T(i, j) = a(i) b(j) (host)

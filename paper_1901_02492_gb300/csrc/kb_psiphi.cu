@@ -556,7 +556,38 @@ __global__ void quantize_kernel(const float2 *__restrict__ f32, pair16 *__restri
     }
 }
 
+// Rows of the padded planes into a contiguous [N][H][W] array on the same device, a CTA per
+// run of a row, 4 elements per thread in flight.  One launch for all epochs: 8 x 1531 x 2047
+// 16-bit codes 28 us, against about 150 as one 2-D copy for each epoch (rows of odd pitch).
+template <typename T>
+__global__ void __launch_bounds__(256) copy_rows_kernel(const T *__restrict__ src, T *__restrict__ dst, int H, int W,
+                                                        int pitch, long long plane_elems) {
+    const int y = blockIdx.y, e = blockIdx.z;
+    const T *s = src + e * plane_elems + (long long)y * pitch;
+    T *d = dst + ((long long)e * H + y) * W;
+    const int x0 = blockIdx.x * 1024 + threadIdx.x;
+    T v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (x0 + 256 * i < W) v[i] = __ldg(s + x0 + 256 * i);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (x0 + 256 * i < W) d[x0 + 256 * i] = v[i];
+}
+
 }  // namespace
+
+cudaError_t launch_copy_rows(const void *src, void *dst, size_t elem, int N, int H, int W, int pitch,
+                             long long plane_elems, cudaStream_t st) {
+    const dim3 grid((W + 1023) / 1024, H, N);
+    if (elem == sizeof(float2))
+        copy_rows_kernel<<<grid, 256, 0, st>>>(static_cast<const float2 *>(src), static_cast<float2 *>(dst), H, W, pitch,
+                                               plane_elems);
+    else
+        copy_rows_kernel<<<grid, 256, 0, st>>>(static_cast<const pair16 *>(src), static_cast<pair16 *>(dst), H, W, pitch,
+                                               plane_elems);
+    return cudaGetLastError();
+}
 
 size_t taps_floats(int N, int K, bool separable) { return (size_t)N * (separable ? 4 * K : 2 * K * K); }
 
