@@ -41,6 +41,7 @@
 //     buffers is full, all its lanes merge theirs in lock step.
 // The Psi/Phi of each kept trajectory are recomputed at the end by the same
 // sequence of operations (bit-identical) together with nobs.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
@@ -442,8 +443,12 @@ __device__ __forceinline__ void add_tail(const E *tab, int n, const L &lane0, co
 // warp's sum) is a chain of a load and six shuffles for every velocity: 12 x 2048^2,
 // 1024 velocities, nu_min 10, psi/phi and bounds included: 8.72 ms that way, 4.10 this way.
 // KEYS: candidate lists in key form for the FP64 rescoring (a.cand_only, k <= kKeyMax).
-template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false>
-__device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4) {
+// SPLIT: the velocities are dealt to the CTAs of a cluster (rank `part` of `parts`, which divides
+// WARPS); each keeps its own lists, then warp w's are brought together by rank w % parts, which
+// reads the others' through distributed shared memory and writes the records.
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false, bool SPLIT = false>
+__device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4,
+                                            int part = 0, int parts = 1) {
     typedef Store<STORAGE> St;
     typedef typename St::T T;         // one pixel's (psi, phi)
     typedef Gather<STORAGE> G;
@@ -558,8 +563,13 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     const int gl = lane & (GL - 1), gs = lane & ~(GL - 1);
     const unsigned gmask = (GL == 32 ? 0xffffffffu : (1u << GL) - 1u) << gs;
     const int vchunk = min(a.V, min(ROWS, TAB / max(NJP, 1)));
-    for (int c0 = 0; c0 < a.V; c0 += vchunk) {
-        const int nc = min(vchunk, a.V - c0);
+    int v0 = 0, v1 = a.V;   // this CTA's velocities, in processing order
+    if constexpr (SPLIT) {
+        v0 = (int)((long long)a.V * part / parts);
+        v1 = (int)((long long)a.V * (part + 1) / parts);
+    }
+    for (int c0 = v0; c0 < v1; c0 += vchunk) {
+        const int nc = min(vchunk, v1 - c0);
         __syncthreads();
         for (int b = warp * (32 / GL); b < nc; b += WARPS * (32 / GL)) {
             const int vi = b + gs / GL;
@@ -661,8 +671,55 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
             if (__any_sync(0xffffffffu, full)) merge_lists();
         }
     }
-    if (!active) return;
-    merge_lists();
+    if constexpr (SPLIT) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        if (active) merge_lists();
+        cluster.sync();   // every CTA's lists are complete
+        if (active && warp % parts == part) {
+            // the other CTAs' lists are sorted: each is read until an entry no longer counts
+#pragma unroll 1
+            for (int q = 0; q < parts; ++q) {
+                if (q == part) continue;
+#pragma unroll
+                for (int p = 0; p < PX; ++p) {
+                    if constexpr (KEYS) {
+                        const uint32_t *rk = cluster.map_shared_rank(lk0 + p * THREADS, q);
+                        uint32_t *lk = lk0 + p * THREADS;
+                        for (int i = 0; i < k; ++i) {
+                            const uint32_t ck = rk[i * LS];
+                            if (ck <= lk[(k - 1) * LS]) break;
+                            int j = k - 1;
+                            for (; j > 0 && lk[(j - 1) * LS] < ck; --j) lk[j * LS] = lk[(j - 1) * LS];
+                            lk[j * LS] = ck;
+                        }
+                    } else {
+                        const float *rn = cluster.map_shared_rank(ln0 + p * THREADS, q);
+                        const uint16_t *rv = cluster.map_shared_rank(lv0 + p * THREADS, q);
+                        float *ln = ln0 + p * THREADS;
+                        uint16_t *lv = lv0 + p * THREADS;
+                        for (int i = 0; i < k; ++i) {
+                            const float cn = rn[i * LS];
+                            const int cv = rv[i * LS];
+                            if (!better(cn, cv, ln[(k - 1) * LS], lv[(k - 1) * LS])) break;
+                            int j = k - 1;
+                            for (; j > 0 && better(cn, cv, ln[(j - 1) * LS], lv[(j - 1) * LS]); --j) {
+                                ln[j * LS] = ln[(j - 1) * LS];
+                                lv[j * LS] = lv[(j - 1) * LS];
+                            }
+                            ln[j * LS] = cn;
+                            lv[j * LS] = (uint16_t)cv;
+                        }
+                    }
+                }
+            }
+        }
+        cluster.sync();   // no CTA leaves, or writes its columns again, before the others have read
+        if (!active || warp % parts != part) return;
+    } else {
+        if (!active) return;
+        merge_lists();
+    }
     if constexpr (KEYS) {
         // candidates for the rescoring, best first, as the keys themselves (4 bytes each,
         // decoded by the rescoring, which recomputes the sums)
@@ -763,7 +820,7 @@ constexpr int min_ctas_batch() {
     return (STORAGE == KB_F32 ? P <= 2 : P <= 1) ? 3 : 2;
 }
 
-template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS>
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, min_ctas<STORAGE, P, C, KM, KEYS>())
     search_kernel(SearchArgs a) {
     __shared__ float2 s_scale[KB_MAX_EPOCHS];
@@ -778,7 +835,9 @@ __global__ void __launch_bounds__(THREADS, min_ctas<STORAGE, P, C, KM, KEYS>())
         by = r / w;
         bx = s * a.swz + (r - by * w);
     }
-    search_tile<STORAGE, P, C, KM, I, PRUNE, KEYS>(a, bx, a.by0 + by, s_scale, s_dyn4);
+    // SPLIT: a cluster is the grid's whole z extent, so z is the CTA's rank in it
+    search_tile<STORAGE, P, C, KM, I, PRUNE, KEYS, SPLIT>(a, bx, a.by0 + by, s_scale, s_dyn4, SPLIT ? blockIdx.z : 0,
+                                                          SPLIT ? gridDim.z : 1);
 }
 
 // Persistent batch search: CTAs take (job, tile) work items from an atomic
@@ -816,13 +875,36 @@ size_t tile_smem(int k) {
                (KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t));
 }
 
+// CTAs (a cluster) that share a tile's velocities: as many of 2, 4 or 8 as leave the launch
+// within one wave of resident CTAs, with at least 16 velocities each.  A launch of a few tiles
+// leaves most SMs idle otherwise: 5 x 64 x 64, 256 velocities is 8 tiles and 171 us, with 8 CTAs
+// per tile 59; beyond one wave the lists' extra work (each CTA fills its own) is not repaid.
+template <int STORAGE, int P, int C, int KM, bool KEYS>
+int split_of(const SearchArgs &a, dim3 grid) {
+    int s = 1;
+    while (s < 8 && (long long)grid.x * grid.y * (2 * s) <= 152LL * min_ctas<STORAGE, P, C, KM, KEYS>() &&
+           a.V >= 16 * (2 * s))
+        s *= 2;
+    return s;
+}
+
 template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false>
 cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
     constexpr int SPAN = 32 * P * Gather<STORAGE>::PIX;
     static_assert(SPAN <= kSpan, "warp span wider than the zero columns");
-    auto kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS>;
     dim3 grid((a.W + SPAN - 1) / SPAN, a.nby > 0 ? a.nby : (a.H + WARPS - 1) / WARPS);
     const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k);
+    // the automatic shapes with 32-bit offsets have a form for small launches
+    constexpr bool kSplit = !PRUNE && sizeof(I) == 4 && KM <= kKeyMax &&
+                            (KEYS || (STORAGE == KB_F32 ? P == 2 && C == 8 : P == 1 && C == 8));
+    int parts = 1;
+    if constexpr (kSplit) {
+        if (a.variant == 0) parts = split_of<STORAGE, P, C, KM, KEYS>(a, grid);
+    }
+    auto kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, false>;
+    if constexpr (kSplit) {
+        if (parts > 1) kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, true>;
+    }
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // Shared-memory carveout: the driver's choice unless the caller sets one
     // (kb_set_search_carveout); it trades resident CTAs against the L1 that the
@@ -830,6 +912,22 @@ cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
     if (err == cudaSuccess && a.carveout >= 0)
         err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, a.carveout);
     if (err != cudaSuccess) return err;
+    if (parts > 1) {
+        grid.z = parts;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = parts;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, a);
+    }
     kern<<<grid, THREADS, smem, st>>>(a);
     return cudaGetLastError();
 }
