@@ -142,15 +142,16 @@ struct kb_job {
     int N = 0, V = 0, k = 0, kkeep = 0;   // kkeep = candidates kept by the search kernel
     int storage = KB_F32;
     bool rescored = false;
-    // device tables
-    int2 *offs = nullptr;        // [Vcap][Ncap] (dx, dy) in time order of epochs
-    int *vorder = nullptr;       // [Vcap] processing order -> caller vidx
-    uint32_t *ptab = nullptr;    // [Vcap][Ncap] producer table, processing order
+    // device tables of the last search, within one block
+    void *tables = nullptr;
+    int2 *offs = nullptr;        // [V][N] (dx, dy) in time order of epochs
+    int *vorder = nullptr;       // [V] processing order -> caller vidx
+    uint32_t *ptab = nullptr;    // [V][N - n0] packed (dx, dy), processing order
     int *status = nullptr;       // device status word of the last search
     int *hstat = nullptr;        // pinned host copies, written after the last search: [0] status, [1] repaired
     cudaEvent_t done = nullptr;  // recorded after the last search's kernels
-    int *epoch_of = nullptr;     // [Ncap] time-order position -> stack epoch
-    float2 *vq = nullptr;        // [Vcap] quantised velocity (px/day) for the results
+    int *epoch_of = nullptr;     // [N] time-order position -> stack epoch
+    float2 *vq = nullptr;        // [V] quantised velocity (px/day) for the results
     // pinned staging for the tables
     void *stage = nullptr;
     size_t stage_bytes = 0, stage_cap = 0;
