@@ -122,7 +122,8 @@ int kb_debug_word(kb_ctx *ctx, unsigned long long *word, int reset);
 /* Tuning hook: force the search kernel used by later kb_search calls of this
  * context; results do not depend on the choice.
  *   0      automatic: the register-gather kernel in its default shape, (2,8) for
- *          FP32 and (1,8) for 16-bit storage ((2,4) for rescoring candidates)
+ *          FP32 and for 16-bit storage (1,4), (1,8) for lists longer than 8 and
+ *          (2,4) for rescoring candidates
  *   1..4   register-gather kernel, (loads per lane, epochs per load batch) =
  *          (4,4), (2,4), (4,8), (2,8) for FP32 and (2,4), (1,4), (2,8), (1,8)
  *          for 16-bit storage, whose loads are pixel pairs

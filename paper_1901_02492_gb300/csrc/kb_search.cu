@@ -227,11 +227,12 @@ struct LaneBase<T, true> {
     }
     __device__ __forceinline__ static uint32_t offset(long long elem) { return (uint32_t)(elem * (long long)sizeof(T)); }
 };
-// Byte offsets where registers are short: FP32 lists up to 8 long, held to 64 (12 x 4096^2,
-// k = 8: 75.8 ms; pointers 80.5, one value of the loop in local memory).  Elsewhere the
-// extra add costs more: BF16 key lists 25.8 ms against 25.5 with pointers (4096 x 2048).
+// Byte offsets where registers are short: value lists up to 8 long, held to 64 (FP32, 12 x
+// 4096^2, k = 8: 75.8 ms; pointers 80.5, one value of the loop in local memory; BF16, 12 x
+// 2048^2, 1024 velocities, (1, 4): 18.6 ms; pointers 21.6).  Elsewhere the extra add costs
+// more: BF16 key lists 25.8 ms against 25.5 with pointers (4096 x 2048).
 template <int STORAGE, int KM, bool KEYS, typename I>
-__host__ __device__ constexpr bool byte_offsets() { return sizeof(I) == 4 && STORAGE == KB_F32 && KM <= kShortMax; }
+__host__ __device__ constexpr bool byte_offsets() { return sizeof(I) == 4 && KM <= kShortMax && !KEYS; }
 
 // Candidate lists of a search that only feeds the FP64 rescoring (KEYS): one
 // 32-bit key per slot.  With b = a.key_bits bits for a velocity index, the high
@@ -896,7 +897,7 @@ cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
     const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k);
     // the automatic shapes with 32-bit offsets have a form for small launches
     constexpr bool kSplit = !PRUNE && sizeof(I) == 4 && KM <= kKeyMax &&
-                            (KEYS || (STORAGE == KB_F32 ? P == 2 && C == 8 : P == 1 && C == 8));
+                            (KEYS || (STORAGE == KB_F32 ? P == 2 && C == 8 : P == 1 && C == (KM > kShortMax ? 8 : 4)));
     int parts = 1;
     if constexpr (kSplit) {
         if (a.variant == 0) parts = split_of<STORAGE, P, C, KM, KEYS>(a, grid);
@@ -961,9 +962,10 @@ cudaError_t launch_idx(const SearchArgs &a, cudaStream_t st) {
 }
 
 // Shapes: (loads per lane P, epochs per load batch C); a 16-bit load is two pixels.
-// Defaults (variant 0): FP32 (2, 8), 12 x 4096^2, k = 8: 76 ms; 16-bit value lists (1, 8),
-// 1500 x 1700, 10 epochs, 500 velocities, BF16 / FP16 at k = 8: 6.32 / 6.26 ms, (1, 4) 6.87 /
-// 6.15, (2, 8) 7.29 / 7.19, (2, 4) 7.52 / 7.49; BF16 at k = 12: 8.40, (1, 4) 9.50, (2, 8) 11.1.
+// Defaults (variant 0): FP32 (2, 8), 12 x 4096^2, k = 8: 76 ms; 16-bit value lists up to 8
+// long (1, 4), 12 x 2048^2, 1024 velocities, k = 8, BF16 / FP16: 18.6 / 18.8 ms, (1, 8) 20.8 /
+// 20.7; longer ones (1, 8), 12 x 1800^2, 1024 velocities, k = 12, BF16: 18.7 ms, (1, 4) 21.9,
+// (2, 4) 20.8, (2, 8) 23.2.
 template <int STORAGE>
 cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
     if constexpr (STORAGE == KB_F32) {
@@ -989,7 +991,7 @@ cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
                 if (use_keys(a)) return launch_keys<STORAGE, 2, 4>(a, st);
                 if (a.snr2)
                     return a.k > kShortMax ? launch_idx<STORAGE, 1, 4, true>(a, st) : launch_idx<STORAGE, 2, 4, true>(a, st);
-                return launch_idx<STORAGE, 1, 8>(a, st);
+                return a.k > kShortMax ? launch_idx<STORAGE, 1, 8>(a, st) : launch_idx<STORAGE, 1, 4>(a, st);
         }
     }
 }
@@ -1099,7 +1101,7 @@ int search_span(int storage, int variant, int k) {
 
 int search_auto_span(int storage, int k) { return search_span(storage, 0, k); }   // of the pruned search
 
-int default_variant(int, int) { return 4; }   // (2, 8), 16-bit (1, 8)
+int default_variant(int storage, int k) { return storage != KB_F32 && k <= kShortMax ? 2 : 4; }   // (1, 4); (2, 8), (1, 8)
 
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
                                 int variant, int kmax, int carve, bool idx64, int sm_count, cudaStream_t st) {
