@@ -498,7 +498,7 @@ typedef struct kb_batch_item {
 /* The plan of one group (filled by kb_batch_groups). */
 typedef struct kb_batch_group {
     int storage;            /* KB_F32 / KB_BF16 / KB_F16 */
-    int index_bits;         /* 32 or 64: width of the element offsets */
+    int index_bits;         /* 32 or 64: width of the offsets in the search's table */
     int variant;            /* tile shape 1..4 (see kb_set_search_variant) */
     int kmax;               /* candidate-list length of its searches */
     long long n_items;      /* CTA tiles in its work list */

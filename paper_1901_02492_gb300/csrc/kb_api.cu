@@ -998,7 +998,7 @@ struct kb_batch {
 
 namespace {
 
-int index_bits(const kb::SearchArgs &a) { return kb::search_idx32(a) ? 32 : 64; }
+int index_bits(const kb::SearchArgs &a) { return kb::search_idx32(a, false) ? 32 : 64; }
 
 // Items of a group for one tile shape: whole searches, or (sample) a band of
 // about `frac` of each search's rows from its middle.

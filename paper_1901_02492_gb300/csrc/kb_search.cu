@@ -108,7 +108,7 @@ using namespace dev;
 constexpr int WARPS = 8;
 constexpr int THREADS = WARPS * 32;
 constexpr uint16_t kNoV = 0xFFFF;   // empty list slot (velocity indices are < 65535)
-constexpr int kShortMax = 8;        // lists up to this long merge in a network of 8,
+// lists up to kShortMax long merge in a network of 8,
 constexpr int kKeyMax = 16;         // up to this (and key lists) in one of 16,
 constexpr int kListMax = 32;        // and all others by walking
 
@@ -944,7 +944,7 @@ cudaError_t launch_one(const SearchArgs &a, cudaStream_t st) {
 // the candidate search of the FP64 rescoring in key form (automatic shape, no pruning)
 template <int STORAGE, int P, int C>
 cudaError_t launch_keys(const SearchArgs &a, cudaStream_t st) {
-    if (search_idx32(a)) return launch_pt<STORAGE, P, C, kKeyMax, int, false, true>(a, st);
+    if (search_idx32(a, true)) return launch_pt<STORAGE, P, C, kKeyMax, int, false, true>(a, st);
     return launch_pt<STORAGE, P, C, kKeyMax, long long, false, true>(a, st);
 }
 
@@ -953,11 +953,11 @@ bool use_keys(const SearchArgs &a) {
     return a.cand_only && !a.snr2 && a.k <= kKeyMax && a.key_bits >= 1 && a.key_bits <= 12;
 }
 
-// 32-bit offsets when every plane of both phases (and the bound planes) fits
+// 32-bit offsets when every plane of both phases (and the bound planes) is in their reach
 template <int STORAGE, int P, int C, bool PRUNE = false>
 cudaError_t launch_idx(const SearchArgs &a, cudaStream_t st) {
     const long long rspan = PRUNE ? (long long)a.N * a.H * ((a.W + 31) / 32 + P * Gather<STORAGE>::PIX) : 0;
-    if (search_idx32(a) && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
+    if (search_idx32(a, false) && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
     return launch_one<STORAGE, P, C, long long, PRUNE>(a, st);
 }
 
