@@ -846,6 +846,7 @@ static int prepare_search(kb_job *job, const kb_stack *s, const double *times, c
     a.status = job->status;
     a.by0 = 0;
     a.nby = 0;
+    a.slots = 0;
     // automatic tile order: super-columns of 8 tiles (12 x 4096^2, FP32, k = 8: 97.7 ms
     // against 117.4 ms row by row; 6 and 12 tiles within 1 %)
     a.swz = ctx->search_swizzle < 0 ? 8 : ctx->search_swizzle;
@@ -1032,9 +1033,12 @@ void make_items(const kb_batch *b, int g, int variant, double frac, std::vector<
 cudaError_t launch_group(const kb_batch *b, int g, int variant, int schedule, int n_items, double frac,
                          cudaStream_t st, cudaStream_t st2) {
     const kb_batch_group &G = b->groups[g];
-    if (schedule == 0)
+    if (schedule == 0) {
+        int njs = 0;
+        for (int j : b->group_jobs[g]) njs = std::max(njs, b->args[j].N - b->args[j].n0);
         return kb::launch_search_batch(b->d_args, b->group_items[g], n_items, b->d_counters + g, G.storage, variant,
-                                       G.kmax, b->ctx->search_carveout, G.index_bits == 64, b->ctx->sm_count, st);
+                                       G.kmax, njs, b->ctx->search_carveout, G.index_bits == 64, b->ctx->sm_count, st);
+    }
     cudaError_t e = cudaSuccess;
     int n = 0;
     for (int j : b->group_jobs[g]) {

@@ -226,6 +226,7 @@ struct SearchArgs {
                              // rescoring recomputes the sums), so the epilogue gathers nothing
     const float *snr2;       // KB_PRUNE: span bound planes [N][H][(W + 31) / 32 + span / 32] (stack epochs), else null
     float nu_min2_slack;     // KB_PRUNE: skip a span when its bound times (1 + 2^-14) is below this (nu_min^2)
+    int slots;               // slots of a list column, k and the buffer's (set by the launch)
 };
 constexpr int kShortMax = 8;   // the longest value lists of the search's short form
 // Whether the search's table holds 32-bit offsets.  Short value lists add byte offsets from the
@@ -244,27 +245,27 @@ template <int STORAGE>
 cudaError_t launch_search_storage(const SearchArgs &a, cudaStream_t st);
 template <int STORAGE>
 cudaError_t launch_search_batch_storage(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int variant,
-                                        int kmax, int carve, bool idx64, int sm_count, cudaStream_t st);
+                                        int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st);
 template <int STORAGE>
 cudaError_t debug_word_storage(unsigned long long *word, bool reset);
 template <>
 cudaError_t launch_search_storage<KB_F32>(const SearchArgs &, cudaStream_t);
 template <>
-cudaError_t launch_search_batch_storage<KB_F32>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+cudaError_t launch_search_batch_storage<KB_F32>(const SearchArgs *, const int4 *, int, int *, int, int, int, int, bool, int,
                                                cudaStream_t);
 template <>
 cudaError_t debug_word_storage<KB_F32>(unsigned long long *, bool);
 template <>
 cudaError_t launch_search_storage<KB_BF16>(const SearchArgs &, cudaStream_t);
 template <>
-cudaError_t launch_search_batch_storage<KB_BF16>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+cudaError_t launch_search_batch_storage<KB_BF16>(const SearchArgs *, const int4 *, int, int *, int, int, int, int, bool, int,
                                                cudaStream_t);
 template <>
 cudaError_t debug_word_storage<KB_BF16>(unsigned long long *, bool);
 template <>
 cudaError_t launch_search_storage<KB_F16>(const SearchArgs &, cudaStream_t);
 template <>
-cudaError_t launch_search_batch_storage<KB_F16>(const SearchArgs *, const int4 *, int, int *, int, int, int, bool, int,
+cudaError_t launch_search_batch_storage<KB_F16>(const SearchArgs *, const int4 *, int, int *, int, int, int, int, bool, int,
                                                cudaStream_t);
 template <>
 cudaError_t debug_word_storage<KB_F16>(unsigned long long *, bool);
@@ -295,7 +296,7 @@ cudaError_t launch_search_tma(const SearchArgs &a, cudaStream_t st);
 // one launch share storage, shape (variant 0..4) and index width; lists sized for kmax;
 // carve = shared-memory carveout percent (-1: the automatic rule)
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
-                                int variant, int kmax, int carve, bool idx64, int sm_count, cudaStream_t st);
+                                int variant, int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st);
 // pixels per CTA row segment of a register-gather shape (tile width) for lists of k
 int search_span(int storage, int variant, int k);
 // the explicit shape (1..4) that the automatic choice (variant 0) takes for lists of k

@@ -45,7 +45,10 @@
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
+#include <stddef.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "kb_device.cuh"
 
@@ -381,7 +384,6 @@ __device__ __forceinline__ void insert_values(float *ln, uint16_t *lv, int k, in
 // for 3 CTAs per SM (FP16, 1500 x 1700, 10 epochs, 500 velocities: (2, 4) 7.52 ms; 4 entries 7.98).
 template <int KM, bool KEYS, int PX>
 __host__ __device__ constexpr int list_cap() { return KEYS ? 4 : KM > kShortMax ? 5 : PX == 4 ? 3 : 4; }
-
 // Adds B epochs (a multiple of four) of one velocity to a lane's sums: every load issued
 // before the first sum, the sums in epoch order.
 template <int STORAGE, int P, int B, typename E, typename T, typename L>
@@ -447,7 +449,8 @@ __device__ __forceinline__ void add_tail(const E *tab, int n, const L &lane0, co
 // SPLIT: the velocities are dealt to the CTAs of a cluster (rank `part` of `parts`, which divides
 // WARPS); each keeps its own lists, then warp w's are brought together by rank w % parts, which
 // reads the others' through distributed shared memory and writes the records.
-template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false, bool SPLIT = false>
+// CUT: the launch shortened the columns' buffers (buffer_cap): a column has a.slots slots.
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS, bool SPLIT, bool CUT>
 __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4,
                                             int part = 0, int parts = 1) {
     typedef Store<STORAGE> St;
@@ -462,18 +465,19 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     constexpr int PX = P * G::PIX;    // pixels per lane
     constexpr int SPAN = 32 * PX;     // pixels per warp row segment
     constexpr int LS = THREADS * PX;  // list columns (pixels) of the CTA
-    constexpr int CAP = list_cap<KM, KEYS, PX>();             // buffer entries of a column
+    constexpr int CAP = list_cap<KM, KEYS, PX>();             // most buffer entries of a column
 
     // s_scale: per time-ordered epoch.  s_dyn4: table E [TAB] | (PRUNE) bound offsets I [TAB] |
-    // velocity ids and entry counts [ROWS] | lists with their buffers: nu float [(k + CAP) * LS],
-    // vidx u16 [(k + CAP) * LS] (KEYS: keys u32 [(k + CAP) * LS]).
+    // velocity ids and entry counts [ROWS] | lists with their buffers: nu float [slots * LS],
+    // vidx u16 [slots * LS] (KEYS: keys u32 [slots * LS]); slots: k and the buffer's.
     E *s_tab = reinterpret_cast<E *>(s_dyn4);
     I *s_rid = reinterpret_cast<I *>(reinterpret_cast<char *>(s_dyn4) + TAB * EB);
     int *s_vid = reinterpret_cast<int *>(s_rid + (PRUNE ? TAB : 0));
     const int N = a.N, n0 = a.n0, NJ = N - n0, k = a.k;
     const int NJP = (NJ + 3) & ~3;   // table row stride: whole groups of four entries
     float *s_ln = reinterpret_cast<float *>(s_vid + ROWS);
-    uint16_t *s_lv = reinterpret_cast<uint16_t *>(s_ln + (k + CAP) * LS);
+    const int slot_end = CUT ? a.slots * LS : (k + CAP) * LS;   // slots of a column, times LS
+    uint16_t *s_lv = reinterpret_cast<uint16_t *>(s_ln + slot_end);
     uint32_t *s_lk = reinterpret_cast<uint32_t *>(s_vid + ROWS);   // KEYS: the lists instead
     for (int j = threadIdx.x; j < N; j += THREADS)
         s_scale[j] = (STORAGE == KB_F32) ? make_float2(1.0f, 1.0f) : exp_scale(scale_exp(a.scales[a.epoch_of[j]]));
@@ -502,7 +506,7 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     int thv[PX];
     uint32_t thk[PX];   // KEYS: the thresholds as keys
     int off[PX];        // the next free buffer slot of the lane's columns, as an offset from slot 0
-    const int off_lim = (k + CAP) * LS;
+    const int off_lim = slot_end;
 #pragma unroll
     for (int p = 0; p < PX; ++p) {
         thn[p] = -INFINITY;
@@ -821,7 +825,7 @@ constexpr int min_ctas_batch() {
     return (STORAGE == KB_F32 ? P <= 2 : P <= 1) ? 3 : 2;
 }
 
-template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS, bool SPLIT>
+template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS, bool SPLIT, bool CUT>
 __global__ void __launch_bounds__(THREADS, min_ctas<STORAGE, P, C, KM, KEYS>())
     search_kernel(SearchArgs a) {
     __shared__ float2 s_scale[KB_MAX_EPOCHS];
@@ -837,17 +841,17 @@ __global__ void __launch_bounds__(THREADS, min_ctas<STORAGE, P, C, KM, KEYS>())
         bx = s * a.swz + (r - by * w);
     }
     // SPLIT: a cluster is the grid's whole z extent, so z is the CTA's rank in it
-    search_tile<STORAGE, P, C, KM, I, PRUNE, KEYS, SPLIT>(a, bx, a.by0 + by, s_scale, s_dyn4, SPLIT ? blockIdx.z : 0,
-                                                          SPLIT ? gridDim.z : 1);
+    search_tile<STORAGE, P, C, KM, I, PRUNE, KEYS, SPLIT, CUT>(a, bx, a.by0 + by, s_scale, s_dyn4,
+                                                               SPLIT ? blockIdx.z : 0, SPLIT ? gridDim.z : 1);
 }
 
 // Persistent batch search: CTAs take (job, tile) work items from an atomic
 // counter until the list is exhausted, copying the item's job descriptor into
 // shared memory first.  The item list is ordered by cost (largest first), so
 // uneven stacks, grids and epoch counts balance across the SMs.
-template <int STORAGE, int P, int C, int KM, typename I>
+template <int STORAGE, int P, int C, int KM, typename I, bool CUT>
 __global__ void __launch_bounds__(THREADS, min_ctas_batch<STORAGE, P>())
-    search_batch_kernel(const SearchArgs *jobs, const int4 *items, int n_items, int *counter) {
+    search_batch_kernel(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int slots) {
     __shared__ float2 s_scale[KB_MAX_EPOCHS];
     __shared__ SearchArgs s_job;
     __shared__ int s_it;
@@ -859,21 +863,87 @@ __global__ void __launch_bounds__(THREADS, min_ctas_batch<STORAGE, P>())
         if (it >= n_items) break;
         const int4 w = items[it];
         for (int i = threadIdx.x; i < (int)(sizeof(SearchArgs) / sizeof(int)); i += THREADS)
-            reinterpret_cast<int *>(&s_job)[i] = reinterpret_cast<const int *>(jobs + w.x)[i];
+            reinterpret_cast<int *>(&s_job)[i] = CUT && i == (int)(offsetof(SearchArgs, slots) / sizeof(int))
+                                                     ? slots
+                                                     : reinterpret_cast<const int *>(jobs + w.x)[i];
         __syncthreads();
-        search_tile<STORAGE, P, C, KM, I, false>(s_job, w.y, w.z, s_scale, s_dyn4);
+        search_tile<STORAGE, P, C, KM, I, false, false, false, CUT>(s_job, w.y, w.z, s_scale, s_dyn4);
         __syncthreads();
     }
 }
 
-// dynamic shared memory of a CTA with lists of k entries: the table, and the lists with their buffers
+// dynamic shared memory of a CTA with lists of k entries and buffers of cap: the table, and the
+// lists with their buffers
 template <int STORAGE, int P, int KM, typename I, bool PRUNE = false, bool KEYS = false>
-size_t tile_smem(int k) {
+size_t tile_smem(int k, int cap) {
     constexpr int PX = P * Gather<STORAGE>::PIX;
     constexpr int TAB = table_entries<STORAGE, I, PRUNE>();
     return (size_t)TAB * (table_entry_bytes<STORAGE, I>() + (PRUNE ? sizeof(I) : 0)) + TAB / 4 * sizeof(int) +
-           (size_t)(k + list_cap<KM, KEYS, PX>()) * THREADS * PX *
+           (size_t)(k + cap) * THREADS * PX *
                (KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t));
+}
+
+// Buffer entries of a launch whose lists are long or keys (njs: its searches' most epochs past the
+// reference time).  The resident CTAs' shared memory takes 100, 132, 164, 196 or 228 KB of an
+// SM's 256, the L1 gets the rest, and the more epochs a velocity has, the more L1 its early
+// epochs need to stay there until the next velocity; the merges that shorter buffers add weigh
+// less by the same measure.  The longest buffer is taken unless a shorter one, no shorter than
+// `least`, brings the CTAs into the next split down or lets another CTA in.  Measured, ms (split
+// in KB, entries):
+//   FP32 k = 16, 5 x 1500^2, 512 velocities: 228, 5: 6.0; 196, 4: 6.7; 12 x 4096^2, 512: 77.5 and 67.2;
+//     20 x 1900^2, 512: 32.9 and 22.1; 24 x 4096^2, 96: 136.6 and 73.1
+//   FP16 k = 16, 12 x 4096^2, 512: 228, 5: 70.0; 196, 3: 76.4; 16 x 1900^2, 512: 19.2 and 19.4;
+//     16 x 4096^2, 96: 47.6 and 37.2; 20 x 1900^2, 512: 24.1 and 21.6; 24 x 4096^2, 96: 102.5 and 57.2
+//   FP32 k = 14, 20 x 1900^2, 512: 196, 5: 20.0; 164, 3: 20.6; 24 x 4096^2, 96: 65.2 and 52.5
+//   FP16 k = 12, 20 x 1900^2, 512: 196, 5: 16.8; 164, 4: 17.0; 24 x 4096^2, 96: 44.9 and 38.9
+//   FP32 k = 9, 20 x 1900^2, 512: 164, 5: 15.9; 132, 4: 16.0; 24 x 4096^2, 96: 36.8 and 34.2
+//   FP16 k = 9, 24 x 4096^2, 96: 164, 5: 31.2; 132, 3: 33.5; 40 x 4096^2, 64: 58.2 and 52.6
+//   BF16 keys, k_c = 12, 4096^2, 24 / 40 / 59: 228, 4: 38.6 / 61.7 / 96.7; 196, 2: 39.7 / 59.0 / 90.9
+//   FP16 candidates, k_c = 20, 12 x 2048^2 / 40 x 4096^2: two CTAs, 5: 27.2 / 154; three, 3: 24.0 / 147
+//     (128 x 1024^2: 34.1 and 35.1)
+// The persistent batch kernel (BATCH), whose searches are mixed, leaves only the 228 KB split in
+// 16-bit storage, above 20 epochs (three searches of 0.5 to 1 M pixels, BF16, k = 16, 8 to 20
+// epochs: 10.2 ms as it is, 12.6 with buffers of 3; 26 to 38 epochs: 25.9 and 20.4).
+template <int STORAGE, int P, int KM, typename I, bool PRUNE, bool KEYS, bool BATCH, typename Kern>
+cudaError_t buffer_cap(Kern kern, int k, int njs, int &cap) {
+    cap = list_cap<KM, KEYS, P * Gather<STORAGE>::PIX>();
+    if (KM <= kShortMax) return cudaSuccess;
+    cudaFuncAttributes fa;
+    cudaError_t err = cudaFuncGetAttributes(&fa, kern);
+    if (err != cudaSuccess) return err;
+    constexpr bool F32 = STORAGE == KB_F32;
+    const size_t KB = 1024, own = fa.sharedSizeBytes + KB;   // each CTA's static share and the system's
+    const int by_regs = 65536 / (((fa.numRegs + 7) & ~7) * THREADS);
+    auto bytes = [&](int c) { return tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(k, c) + own; };
+    auto ctas = [&](int c) { return std::min(by_regs, (int)(228 * KB / bytes(c))); };
+    auto split = [&](int c) {
+        const size_t all = ctas(c) * bytes(c);
+        for (int kb = 100; kb < 228; kb += 32)
+            if (all <= kb * KB) return kb;
+        return 228;
+    };
+    auto least = [&](int from) {   // the shortest buffer that is worth leaving a split
+        constexpr int none = 99;
+        if (KEYS) return from == 228 && njs > 32 ? 2 : none;
+        if (BATCH && !F32) return from == 228 && njs > 20 ? 2 : none;
+        if (njs <= 20 && from == 228) return njs <= 8 ? none : njs <= 12 ? 4 : 3;
+        if (from == 228) return 2;
+        if (njs <= 20) return none;
+        if (from == 196) return F32 || njs > 48 ? 2 : 3;
+        return F32 ? (njs <= 32 ? 4 : 3) : njs <= 48 ? none : 3;
+    };
+    for (int c = cap - 1; c >= 2; --c) {
+        if (ctas(c) > ctas(cap) ? c >= 3 && njs <= 64 : ctas(c) == ctas(cap) && split(c) < split(cap) && c >= least(split(cap)))
+            cap = c;
+    }
+    return cudaSuccess;
+}
+
+// the shapes of the automatic choice (launch_storage): they have a kernel for buffers of their full
+// length, a constant, and one whose slots come with the launch (which takes BF16 3 % longer)
+template <int STORAGE, int P, int C, int KM, bool PRUNE, bool KEYS>
+constexpr bool auto_shape() {
+    return !PRUNE && (KEYS || (STORAGE == KB_F32 ? P == 2 && C == 8 : P == 1 && C == (KM > kShortMax ? 8 : 4)));
 }
 
 // CTAs (a cluster) that share a tile's velocities: as many of 2, 4 or 8 as leave the launch
@@ -889,24 +959,39 @@ int split_of(const SearchArgs &a, dim3 grid) {
     return s;
 }
 
+// the other shapes' kernels for long lists: with the launch's slots, but for wide 16-bit ones,
+// whose CTAs are one or two per SM either way
+template <int STORAGE, int P, int KM>
+constexpr bool always_cut() { return KM > kShortMax && (STORAGE == KB_F32 || P == 1); }
+
 template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS = false>
-cudaError_t launch_pt(const SearchArgs &a, cudaStream_t st) {
+cudaError_t launch_pt(const SearchArgs &search, cudaStream_t st) {
+    SearchArgs a = search;
     constexpr int SPAN = 32 * P * Gather<STORAGE>::PIX;
     static_assert(SPAN <= kSpan, "warp span wider than the zero columns");
     dim3 grid((a.W + SPAN - 1) / SPAN, a.nby > 0 ? a.nby : (a.H + WARPS - 1) / WARPS);
-    const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k);
+    constexpr bool kAuto = auto_shape<STORAGE, P, C, KM, PRUNE, KEYS>(), kLong = KM > kShortMax;
     // the automatic shapes with 32-bit offsets have a form for small launches
-    constexpr bool kSplit = !PRUNE && sizeof(I) == 4 && KM <= kKeyMax &&
-                            (KEYS || (STORAGE == KB_F32 ? P == 2 && C == 8 : P == 1 && C == (KM > kShortMax ? 8 : 4)));
-    int parts = 1;
+    constexpr bool kSplit = kAuto && sizeof(I) == 4 && KM <= kKeyMax;
+    constexpr int CAP = list_cap<KM, KEYS, P * Gather<STORAGE>::PIX>();
+    int parts = 1, cap = CAP;
     if constexpr (kSplit) {
         if (a.variant == 0) parts = split_of<STORAGE, P, C, KM, KEYS>(a, grid);
     }
-    auto kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, false>;
-    if constexpr (kSplit) {
-        if (parts > 1) kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, true>;
+    constexpr bool kCut = !kAuto && always_cut<STORAGE, P, KM>();
+    auto kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, false, kCut>;
+    cudaError_t err = cudaSuccess;
+    if (parts == 1 && (kAuto || kCut)) err = buffer_cap<STORAGE, P, KM, I, PRUNE, KEYS, false>(kern, a.k, a.N - a.n0, cap);
+    if (err != cudaSuccess) return err;
+    if constexpr (kLong && kAuto) {
+        if (cap < CAP) kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, false, true>;
     }
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if constexpr (kSplit) {
+        if (parts > 1) kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, true, false>;
+    }
+    a.slots = a.k + cap;
+    const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k, cap);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // Shared-memory carveout: the driver's choice unless the caller sets one
     // (kb_set_search_carveout); it trades resident CTAs against the L1 that the
     // early epochs' gathers reuse across velocities.
@@ -998,10 +1083,20 @@ cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
 
 template <int STORAGE, int P, int C, int KM, typename I>
 cudaError_t launch_batch_pt(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int kmax,
-                            int carve, int sm_count, cudaStream_t st) {
-    const size_t smem = tile_smem<STORAGE, P, KM, I>(kmax);
-    auto kern = search_batch_kernel<STORAGE, P, C, KM, I>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                            int njs, int carve, int sm_count, cudaStream_t st) {
+    constexpr bool kAuto = auto_shape<STORAGE, P, C, KM, false, false>(), kLong = KM > kShortMax;
+    constexpr int CAP = list_cap<KM, false, P * Gather<STORAGE>::PIX>();
+    constexpr bool kCut = !kAuto && always_cut<STORAGE, P, KM>();
+    auto kern = search_batch_kernel<STORAGE, P, C, KM, I, kCut>;
+    int cap = CAP;
+    cudaError_t err = cudaSuccess;
+    if (kAuto || kCut) err = buffer_cap<STORAGE, P, KM, I, false, false, true>(kern, kmax, njs, cap);
+    if (err != cudaSuccess) return err;
+    if constexpr (kLong && kAuto) {
+        if (cap < CAP) kern = search_batch_kernel<STORAGE, P, C, KM, I, true>;
+    }
+    const size_t smem = tile_smem<STORAGE, P, KM, I>(kmax, cap);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err == cudaSuccess && carve >= 0)
         err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
     int per_sm = 0;
@@ -1009,44 +1104,44 @@ cudaError_t launch_batch_pt(const SearchArgs *jobs, const int4 *items, int n_ite
     if (err != cudaSuccess) return err;
     // persistent grid: every SM filled with as many CTAs as it can hold
     const int grid = sm_count * (per_sm > 0 ? per_sm : 1);
-    kern<<<grid, THREADS, smem, st>>>(jobs, items, n_items, counter);
+    kern<<<grid, THREADS, smem, st>>>(jobs, items, n_items, counter, kmax + cap);
     return cudaGetLastError();
 }
 
 template <int STORAGE, int P, int C, typename I>
 cudaError_t launch_batch_one(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int kmax,
-                             int carve, int sm_count, cudaStream_t st) {
+                             int njs, int carve, int sm_count, cudaStream_t st) {
     if (kmax > kKeyMax)
-        return launch_batch_pt<STORAGE, P, C, kListMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+        return launch_batch_pt<STORAGE, P, C, kListMax, I>(jobs, items, n_items, counter, kmax, njs, carve, sm_count, st);
     if (kmax > kShortMax)
-        return launch_batch_pt<STORAGE, P, C, kKeyMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
-    return launch_batch_pt<STORAGE, P, C, kShortMax, I>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+        return launch_batch_pt<STORAGE, P, C, kKeyMax, I>(jobs, items, n_items, counter, kmax, njs, carve, sm_count, st);
+    return launch_batch_pt<STORAGE, P, C, kShortMax, I>(jobs, items, n_items, counter, kmax, njs, carve, sm_count, st);
 }
 
 template <int STORAGE, int P, int C>
 cudaError_t launch_batch_idx(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int kmax,
-                             int carve, bool idx64, int sm_count, cudaStream_t st) {
+                             int njs, int carve, bool idx64, int sm_count, cudaStream_t st) {
     if (idx64)
-        return launch_batch_one<STORAGE, P, C, long long>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
-    return launch_batch_one<STORAGE, P, C, int>(jobs, items, n_items, counter, kmax, carve, sm_count, st);
+        return launch_batch_one<STORAGE, P, C, long long>(jobs, items, n_items, counter, kmax, njs, carve, sm_count, st);
+    return launch_batch_one<STORAGE, P, C, int>(jobs, items, n_items, counter, kmax, njs, carve, sm_count, st);
 }
 
 template <int STORAGE>
 cudaError_t launch_batch_storage(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int variant,
-                                 int kmax, int carve, bool idx64, int sm_count, cudaStream_t st) {
+                                 int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st) {
     if constexpr (STORAGE == KB_F32) {
         switch (variant) {
-            case 1: return launch_batch_idx<STORAGE, 4, 4>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            case 2: return launch_batch_idx<STORAGE, 2, 4>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            case 3: return launch_batch_idx<STORAGE, 4, 8>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            default: return launch_batch_idx<STORAGE, 2, 8>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
+            case 1: return launch_batch_idx<STORAGE, 4, 4>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            case 2: return launch_batch_idx<STORAGE, 2, 4>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            case 3: return launch_batch_idx<STORAGE, 4, 8>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            default: return launch_batch_idx<STORAGE, 2, 8>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
         }
     } else {
         switch (variant) {
-            case 2: return launch_batch_idx<STORAGE, 1, 4>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            case 3: return launch_batch_idx<STORAGE, 2, 8>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            case 4: return launch_batch_idx<STORAGE, 1, 8>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
-            default: return launch_batch_idx<STORAGE, 2, 4>(jobs, items, n_items, counter, kmax, carve, idx64, sm_count, st);
+            case 2: return launch_batch_idx<STORAGE, 1, 4>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            case 3: return launch_batch_idx<STORAGE, 2, 8>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            case 4: return launch_batch_idx<STORAGE, 1, 8>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
+            default: return launch_batch_idx<STORAGE, 2, 4>(jobs, items, n_items, counter, kmax, njs, carve, idx64, sm_count, st);
         }
     }
 }
@@ -1059,9 +1154,9 @@ cudaError_t launch_search_storage<KB_SEARCH_STORAGE>(const SearchArgs &a, cudaSt
 }
 template <>
 cudaError_t launch_search_batch_storage<KB_SEARCH_STORAGE>(const SearchArgs *jobs, const int4 *items, int n_items,
-                                                           int *counter, int variant, int kmax, int carve, bool idx64,
+                                                           int *counter, int variant, int kmax, int njs, int carve, bool idx64,
                                                            int sm_count, cudaStream_t st) {
-    return launch_batch_storage<KB_SEARCH_STORAGE>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+    return launch_batch_storage<KB_SEARCH_STORAGE>(jobs, items, n_items, counter, variant, kmax, njs, carve, idx64, sm_count, st);
 }
 template <>
 cudaError_t debug_word_storage<KB_SEARCH_STORAGE>(unsigned long long *word, bool reset) {
@@ -1104,11 +1199,11 @@ int search_auto_span(int storage, int k) { return search_span(storage, 0, k); } 
 int default_variant(int storage, int k) { return storage != KB_F32 && k <= kShortMax ? 2 : 4; }   // (1, 4); (2, 8), (1, 8)
 
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
-                                int variant, int kmax, int carve, bool idx64, int sm_count, cudaStream_t st) {
+                                int variant, int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st) {
     switch (storage) {
-        case KB_F32: return launch_search_batch_storage<KB_F32>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
-        case KB_BF16: return launch_search_batch_storage<KB_BF16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
-        case KB_F16: return launch_search_batch_storage<KB_F16>(jobs, items, n_items, counter, variant, kmax, carve, idx64, sm_count, st);
+        case KB_F32: return launch_search_batch_storage<KB_F32>(jobs, items, n_items, counter, variant, kmax, njs, carve, idx64, sm_count, st);
+        case KB_BF16: return launch_search_batch_storage<KB_BF16>(jobs, items, n_items, counter, variant, kmax, njs, carve, idx64, sm_count, st);
+        case KB_F16: return launch_search_batch_storage<KB_F16>(jobs, items, n_items, counter, variant, kmax, njs, carve, idx64, sm_count, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -198,3 +198,33 @@ def test_streaming_images_equal_the_tile_kernel(kb, ctx, N, H, W, K):
             got.append(h)
         s.free()
     assert np.array_equal(got[0], got[2]) and np.array_equal(got[1], got[3])
+
+
+# epochs on both sides of the steps of the buffers' rule (13, 17 and 33 past the reference time, and 65), list
+# lengths whose lists leave buffers of 5, 4, 3 and 2 entries there
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("N", [12, 15, 24, 34, 66])
+def test_buffers_by_the_number_of_epochs(kb, ctx, storage, N):
+    """Long lists (15 and 20 of them rescoring candidates) and key lists, whose buffers shorten with the epochs."""
+    st = synth.small_stack(300 + N, N, 17, 130, K=5, nan_frac=0.02, n_angles=10, n_speeds=13, s_hi=60.0, n_sources=3,
+                           flux=40.0)
+    s, f = _stack(kb, ctx, st, storage), _stack(kb, ctx, st, "f32")
+    for k in (9, 12, 14, 15, 16):
+        ctx.set_search_variant(5)
+        ref = _records(kb, ctx, s, st, 130, k).tobytes()
+        for variant in (0, 4):
+            ctx.set_search_variant(variant)
+            assert _records(kb, ctx, s, st, 130, k).tobytes() == ref, (k, variant)
+        ctx.set_search_variant(0)
+        job = kb.Job(ctx, 17, 130, N, 130, k)
+        batch = kb.Batch(ctx, [dict(job=job, stack=s, times=st.times, vx=st.vx, vy=st.vy, topk=k)], autotune=False)
+        batch.run()
+        assert job.results().tobytes() == ref, k
+        torch.cuda.synchronize()
+        batch.free()
+        job.free()
+    for k in (8, 12, 16):
+        got = _records(kb, ctx, s, st, 130, k, flags=kb.KB_RESCORE_FP64)
+        assert got.tobytes() == _records(kb, ctx, f, st, 130, k, flags=kb.KB_RESCORE_FP64).tobytes(), k
+    for o in (s, f):
+        o.free()
