@@ -234,8 +234,8 @@ constexpr int kShortMax = 8;   // the longest value lists of the search's short 
 // lists add element offsets to a pointer, which reach 2^31 elements.  64-bit entries are twice as
 // large: 40 x 4096^2, 96 velocities, BF16, lists of 12: 101.5 ms with 32-bit offsets, 103.1 with
 // 64-bit ones; 59 epochs, 48 velocities: 145.3 against 147.9.
-inline bool search_idx32(const SearchArgs &a, bool keys) {
-    if (keys || a.k > kShortMax) return a.planes_elems < (1LL << 31) - 1;
+inline bool search_idx32(const SearchArgs &a, bool elements) {
+    if (elements || a.k > kShortMax) return a.planes_elems < (1LL << 31) - 1;
     return a.planes_elems * (a.storage == KB_F32 ? (long long)sizeof(float2) : (long long)sizeof(pair16)) < (1LL << 32);
 }
 // register-gather kernel (variant 0 = its default shape, 1..4)

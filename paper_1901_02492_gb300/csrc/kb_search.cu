@@ -195,6 +195,18 @@ template <int STORAGE, typename I, bool PRUNE>
 __host__ __device__ constexpr int table_entries() {
     return (int)((STORAGE == KB_F32 && !PRUNE ? 2048 : 4096) / table_entry_bytes<STORAGE, I>());
 }
+// The pruned FP32 search with short lists has a form for more than kPruneMany epochs past the
+// reference time, where a bound is a long sum and most of a chunk's lanes have none:
+//   - buffers of 2 (k = 8), so that 4 CTAs stay within the 164 KB split (92 KB of L1, not 60);
+//   - the lanes of a warp share the chunk's velocities, and a sum ends once it reaches nu_min^2;
+//   - the bound offsets' rows have an odd stride (at 64 epochs, 16 lanes otherwise meet in a bank);
+//   - element offsets from a pointer, so that 32-bit ones reach 2^31 elements.
+// 64 x 1024^2, 256 velocities, k = 8, nu_min 5 / 12 / 20: 8.42 / 8.25 / 6.82 ms without it, 6.97 /
+// 7.06 / 5.94 with it; 40 x 4096^2, 96 velocities, nu_min 12: 26.9 and 23.5; 32 x 1024^2, nu_min 20:
+// 0.43 and 0.42; 24 x 1024^2, nu_min 12 / 20: 1.71 / 0.37 and 1.62 / 0.43.
+constexpr int kPruneMany = 28;
+template <int STORAGE, int KM, bool PRUNE, bool CUT>
+__host__ __device__ constexpr bool many_epochs() { return STORAGE == KB_F32 && PRUNE && CUT && KM <= kShortMax; }
 template <typename I>
 __device__ __forceinline__ uint32_t entry_sc(const Entry<I, false> &) { return 0u; }
 template <typename I>
@@ -449,7 +461,8 @@ __device__ __forceinline__ void add_tail(const E *tab, int n, const L &lane0, co
 // SPLIT: the velocities are dealt to the CTAs of a cluster (rank `part` of `parts`, which divides
 // WARPS); each keeps its own lists, then warp w's are brought together by rank w % parts, which
 // reads the others' through distributed shared memory and writes the records.
-// CUT: the launch shortened the columns' buffers (buffer_cap): a column has a.slots slots.
+// CUT: the launch shortened the columns' buffers (buffer_cap): a column has a.slots slots.  With
+// PRUNE, FP32 and short lists also the form for many epochs (MANY, many_epochs()).
 template <int STORAGE, int P, int C, int KM, typename I, bool PRUNE, bool KEYS, bool SPLIT, bool CUT>
 __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by, float2 *s_scale, int4 *s_dyn4,
                                             int part = 0, int parts = 1) {
@@ -460,21 +473,24 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     typedef Entry<I, STORAGE != KB_F32> E;
     static_assert(C % 4 == 0, "entries are read four at a time");
     static_assert(WARPS <= kPadRows, "a band of warps' rows must fit the planes' zero rows");
+    constexpr bool MANY = many_epochs<STORAGE, KM, PRUNE, CUT>();
     constexpr int TAB = table_entries<STORAGE, I, PRUNE>(), ROWS = TAB / 4;
+    constexpr int RID = PRUNE ? TAB + (MANY ? ROWS : 0) : 0;   // bound offsets
     constexpr size_t EB = table_entry_bytes<STORAGE, I>();
     constexpr int PX = P * G::PIX;    // pixels per lane
     constexpr int SPAN = 32 * PX;     // pixels per warp row segment
     constexpr int LS = THREADS * PX;  // list columns (pixels) of the CTA
     constexpr int CAP = list_cap<KM, KEYS, PX>();             // most buffer entries of a column
 
-    // s_scale: per time-ordered epoch.  s_dyn4: table E [TAB] | (PRUNE) bound offsets I [TAB] |
+    // s_scale: per time-ordered epoch.  s_dyn4: table E [TAB] | (PRUNE) bound offsets I [RID] |
     // velocity ids and entry counts [ROWS] | lists with their buffers: nu float [slots * LS],
     // vidx u16 [slots * LS] (KEYS: keys u32 [slots * LS]); slots: k and the buffer's.
     E *s_tab = reinterpret_cast<E *>(s_dyn4);
     I *s_rid = reinterpret_cast<I *>(reinterpret_cast<char *>(s_dyn4) + TAB * EB);
-    int *s_vid = reinterpret_cast<int *>(s_rid + (PRUNE ? TAB : 0));
+    int *s_vid = reinterpret_cast<int *>(s_rid + RID);
     const int N = a.N, n0 = a.n0, NJ = N - n0, k = a.k;
     const int NJP = (NJ + 3) & ~3;   // table row stride: whole groups of four entries
+    const int NJR = MANY ? NJ | 1 : NJP;   // bound offsets' row stride
     float *s_ln = reinterpret_cast<float *>(s_vid + ROWS);
     const int slot_end = CUT ? a.slots * LS : (k + CAP) * LS;   // slots of a column, times LS
     uint16_t *s_lv = reinterpret_cast<uint16_t *>(s_ln + slot_end);
@@ -498,7 +514,7 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     const T *planes = reinterpret_cast<const T *>(a.planes);
     // element index of this lane's first pixel within a plane (even for 16-bit storage)
     const long long tb = a.origin + (long long)y * a.pitch + xw + lane * G::PIX;
-    typedef LaneBase<T, byte_offsets<STORAGE, KM, KEYS, I>()> LB;
+    typedef LaneBase<T, byte_offsets<STORAGE, KM, KEYS, I>() && !MANY> LB;
     const LB lane0(planes, tb);
     const unsigned lt_mask = (1u << lane) - 1u;
 
@@ -568,6 +584,12 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
     const int gl = lane & (GL - 1), gs = lane & ~(GL - 1);
     const unsigned gmask = (GL == 32 ? 0xffffffffu : (1u << GL) - 1u) << gs;
     const int vchunk = min(a.V, min(ROWS, TAB / max(NJP, 1)));
+    // velocities whose bounds are taken at once, 32; MANY: the power of two that holds a chunk, and
+    // 32 / bv lanes share a velocity's epochs
+    int bv = 32;
+    if constexpr (MANY) {
+        while (bv / 2 >= vchunk) bv /= 2;
+    }
     int v0 = 0, v1 = a.V;   // this CTA's velocities, in processing order
     if constexpr (SPLIT) {
         v0 = (int)((long long)a.V * part / parts);
@@ -601,7 +623,7 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
                     if constexpr (STORAGE != KB_F32) e.sc = sc_of(s_scale[j]);
                     s_tab[at] = e;
                     if constexpr (PRUNE)   // the CTA's first row; a warp adds warp * RW
-                        s_rid[at] = (I)(((long long)ep * a.H + y0 + oy) * RW + ((xw + ox) >> 5) + SPAN / 32);
+                        s_rid[at + vi * (NJR - NJP)] = (I)(((long long)ep * a.H + y0 + oy) * RW + ((xw + ox) >> 5) + SPAN / 32);
                 }
                 cnt += __popc(m);
             }
@@ -614,18 +636,39 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
             if constexpr (PRUNE) {
                 if ((vi & 31) == 0) {
                     // a lane's velocity: its span's bound on nu^2, every step rounded upwards
-                    const int mine = vi + lane;
-                    float b = b0;
+                    const int mine = vi + (MANY ? lane & (bv - 1) : lane);
+                    float b = !MANY || lane < bv ? b0 : 0.0f;
                     if (mine < nc) {
-                        const I *rid = s_rid + mine * NJP;
+                        const I *rid = s_rid + mine * NJR;
                         const int n = s_vid[mine] >> 16;
+                        if constexpr (MANY) {
+                            // a bound that has reached nu_min^2 says no more: four epochs, then a look
+                            const int by = 32 / bv;
+                            for (int jj = lane / bv; jj < n && __fmul_ru(b, 1.0f + 0x1p-14f) < a.nu_min2_slack; jj += 4 * by) {
+                                float r4[4];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    r4[u] = 0.0f;
+                                    if (jj + u * by < n) {
+                                        const long long r = rid[jj + u * by] + (long long)warp * RW;
+                                        r4[u] = __ldg(a.snr2 + max(0LL, min(RE - 1, r)));
+                                    }
+                                }
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) b = __fadd_ru(b, r4[u]);
+                            }
+                        } else {
 #pragma unroll 4
-                        for (int jj = 0; jj < n; ++jj) {
-                            const long long r = rid[jj] + (long long)warp * RW;
-                            b = __fadd_ru(b, __ldg(a.snr2 + max(0LL, min(RE - 1, r))));
+                            for (int jj = 0; jj < n; ++jj) {
+                                const long long r = rid[jj] + (long long)warp * RW;
+                                b = __fadd_ru(b, __ldg(a.snr2 + max(0LL, min(RE - 1, r))));
+                            }
                         }
                     }
-                    todo = __ballot_sync(0xffffffffu, mine < nc && !(__fmul_ru(b, 1.0f + 0x1p-14f) < a.nu_min2_slack));
+                    if constexpr (MANY) {
+                        for (int o = bv; o < 32; o *= 2) b = __fadd_ru(b, __shfl_xor_sync(0xffffffffu, b, o));
+                    }
+                    todo = __ballot_sync(0xffffffffu, (!MANY || lane < bv) && mine < nc && !(__fmul_ru(b, 1.0f + 0x1p-14f) < a.nu_min2_slack));
                 }
                 const unsigned rest = todo >> (vi & 31);
                 if (rest == 0u) {
@@ -874,11 +917,11 @@ __global__ void __launch_bounds__(THREADS, min_ctas_batch<STORAGE, P>())
 
 // dynamic shared memory of a CTA with lists of k entries and buffers of cap: the table, and the
 // lists with their buffers
-template <int STORAGE, int P, int KM, typename I, bool PRUNE = false, bool KEYS = false>
+template <int STORAGE, int P, int KM, typename I, bool PRUNE = false, bool KEYS = false, bool MANY = false>
 size_t tile_smem(int k, int cap) {
     constexpr int PX = P * Gather<STORAGE>::PIX;
-    constexpr int TAB = table_entries<STORAGE, I, PRUNE>();
-    return (size_t)TAB * (table_entry_bytes<STORAGE, I>() + (PRUNE ? sizeof(I) : 0)) + TAB / 4 * sizeof(int) +
+    constexpr int TAB = table_entries<STORAGE, I, PRUNE>(), RID = PRUNE ? TAB + (MANY ? TAB / 4 : 0) : 0;
+    return (size_t)TAB * table_entry_bytes<STORAGE, I>() + RID * sizeof(I) + TAB / 4 * sizeof(int) +
            (size_t)(k + cap) * THREADS * PX *
                (KEYS ? sizeof(uint32_t) : sizeof(float) + sizeof(uint16_t));
 }
@@ -989,8 +1032,17 @@ cudaError_t launch_pt(const SearchArgs &search, cudaStream_t st) {
     if constexpr (kSplit) {
         if (parts > 1) kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, true, false>;
     }
+    size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k, cap);
+    if constexpr (many_epochs<STORAGE, KM, PRUNE, true>()) {
+        if (a.N - a.n0 > kPruneMany) {
+            // 4 CTAs (and the system's 1 KB of each) within the 164 KB split of shared memory
+            kern = search_kernel<STORAGE, P, C, KM, I, PRUNE, KEYS, false, true>;
+            do
+                smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS, true>(a.k, cap);
+            while (smem > 40 * 1024 && --cap > 1);
+        }
+    }
     a.slots = a.k + cap;
-    const size_t smem = tile_smem<STORAGE, P, KM, I, PRUNE, KEYS>(a.k, cap);
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // Shared-memory carveout: the driver's choice unless the caller sets one
     // (kb_set_search_carveout); it trades resident CTAs against the L1 that the
@@ -1042,7 +1094,8 @@ bool use_keys(const SearchArgs &a) {
 template <int STORAGE, int P, int C, bool PRUNE = false>
 cudaError_t launch_idx(const SearchArgs &a, cudaStream_t st) {
     const long long rspan = PRUNE ? (long long)a.N * a.H * ((a.W + 31) / 32 + P * Gather<STORAGE>::PIX) : 0;
-    if (search_idx32(a, false) && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
+    const bool elements = PRUNE && STORAGE == KB_F32 && a.k <= kShortMax && a.N - a.n0 > kPruneMany;   // MANY
+    if (search_idx32(a, elements) && rspan < (1LL << 31) - 1) return launch_one<STORAGE, P, C, int, PRUNE>(a, st);
     return launch_one<STORAGE, P, C, long long, PRUNE>(a, st);
 }
 

@@ -228,3 +228,16 @@ def test_buffers_by_the_number_of_epochs(kb, ctx, storage, N):
         assert got.tobytes() == _records(kb, ctx, f, st, 130, k, flags=kb.KB_RESCORE_FP64).tobytes(), k
     for o in (s, f):
         o.free()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("N,V", [(29, 70), (30, 70), (33, 70), (64, 40), (66, 33), (100, 21), (128, 40), (128, 3), (35, 1)])
+def test_pruning_with_many_epochs(kb, ctx, storage, N, V):
+    """Fewer than 32 velocities in a chunk of the table: several lanes share a velocity's bound."""
+    st = synth.small_stack(500 + N, N, 19, 200, K=5, nan_frac=0.02, n_angles=10, n_speeds=10, s_hi=60.0, n_sources=6,
+                           flux=60.0)
+    s = _stack(kb, ctx, st, storage)
+    for k, nu_min in ((1, 4.0), (4, 5.0), (8, 9.0), (10, 9.0)):
+        ref = _records(kb, ctx, s, st, V, k, nu_min)
+        assert _records(kb, ctx, s, st, V, k, nu_min, kb.KB_PRUNE).tobytes() == ref.tobytes()
+    s.free()
