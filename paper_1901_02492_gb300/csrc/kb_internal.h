@@ -351,6 +351,7 @@ struct FilterArgs {
     int krec, k;
     double nsigma2;          // nsigma^2
     kb_filtered *out;        // device [H*W][k]
+    int strip, parts;        // width of a strip, CTAs of its row (set by the launch)
 };
 cudaError_t launch_filter(const FilterArgs &a, cudaStream_t st);
 

@@ -24,6 +24,8 @@
 #include <math.h>
 #include <stddef.h>
 
+#include <algorithm>
+
 #include "kb_internal.h"
 
 namespace kb {
@@ -552,13 +554,14 @@ __global__ void __launch_bounds__(kFilterThreads) filter_kernel(FilterArgs a) {
         s_plane[j] = (long long)a.epoch_of[j] * a.plane_elems + a.origin;
     __syncthreads();
     // the CTA's 128 records of one row of a strip: strips side by side, rows down each
-    const int parts = kStrip * a.k / kFilterThreads, per = parts * a.H;
-    const int strip = blockIdx.x / per, r = blockIdx.x - strip * per, y = r / parts;
-    const int i = (r - y * parts) * kFilterThreads + threadIdx.x;   // record within the strip's row
-    const int px = i / a.k, x = strip * kStrip + px;
-    const long long row = ((long long)y * a.W + strip * kStrip) * a.k;   // its first record
+    const int per = a.parts * a.H;
+    const int strip = blockIdx.x / per, r = blockIdx.x - strip * per, y = r / a.parts;
+    const int i = (r - y * a.parts) * kFilterThreads + threadIdx.x;   // record within the strip's row
+    const int x0 = strip * a.strip, width = min(a.strip, a.W - x0);
+    const int px = i / a.k, x = x0 + px;
+    const long long row = ((long long)y * a.W + x0) * a.k;   // its first record
     const int slot = i - px * a.k;
-    const bool valid = x < a.W;
+    const bool valid = px < width;
     const long long pix = (long long)y * a.W + x;
     uint32_t v = kEmptyVidx;
     if (valid) v = a.recs64 ? a.recs64[pix * a.k + slot].vidx : (a.recs[pix * a.krec + slot].meta & 0xffffu);
@@ -669,17 +672,21 @@ __global__ void __launch_bounds__(kFilterThreads) filter_kernel(FilterArgs a) {
     for (int c = 0; c < 4; ++c)
         w[lane * kWords + 5 + c] = make_uint2((uint32_t)__double2loint(tail[c]), (uint32_t)__double2hiint(tail[c]));
     __syncwarp();
-    const int n = min(32, (min(kStrip, a.W - strip * kStrip)) * a.k - (i - lane));   // records in the image
+    const int n = min(32, width * a.k - (i - lane));   // records in the strip
     uint2 *out = reinterpret_cast<uint2 *>(a.out + row + (i - lane));
     for (int c = lane; c < n * kWords; c += 32) out[c] = w[c];
 }
 
-cudaError_t launch_filter(const FilterArgs &a, cudaStream_t st) {
-    // kStrip * k records of a strip's row are whole CTAs
-    static_assert(kStrip % kFilterThreads == 0, "a strip's row is a whole number of CTAs");
-    const long long blocks = (long long)((a.W + kStrip - 1) / kStrip) * (kStrip * a.k / kFilterThreads) * a.H;
+cudaError_t launch_filter(const FilterArgs &args, cudaStream_t st) {
+    FilterArgs a = args;
+    // strips of kStrip or the image's width, a strip's row in whole CTAs (with strips of 256 whatever the
+    // image, 12 x 2000 x 1, k = 8: 43 us, as 1 thread in 256 had a record, against 23; 5 x 64 x 64,
+    // k = 4: 23 against 19)
+    a.strip = std::min(kStrip, a.W);
+    const int strips = (a.W + a.strip - 1) / a.strip;
+    a.parts = (a.strip * a.k + kFilterThreads - 1) / kFilterThreads;
+    const long long blocks = (long long)strips * a.parts * a.H;   // at most 2^27, for sides up to 32767 and k up to 16
     if (blocks <= 0) return cudaSuccess;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     if (a.N <= 16)
         filter_kernel<16><<<(int)blocks, kFilterThreads, 0, st>>>(a);
     else if (a.N <= 32)

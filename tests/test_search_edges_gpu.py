@@ -241,3 +241,24 @@ def test_pruning_with_many_epochs(kb, ctx, storage, N, V):
         ref = _records(kb, ctx, s, st, V, k, nu_min)
         assert _records(kb, ctx, s, st, V, k, nu_min, kb.KB_PRUNE).tobytes() == ref.tobytes()
     s.free()
+
+
+@pytest.mark.parametrize("N,H,W,k", [(3, 40, 1, 1), (5, 11, 2, 16), (4, 3, 256, 7), (4, 5, 257, 5), (20, 4, 511, 3), (6, 2, 513, 9)])
+def test_filter_on_strips_of_any_width(kb, ctx, N, H, W, k):
+    """Images narrower than a strip, and wider ones that leave a ragged strip: with nothing rejected
+    the filter returns the search's own trajectories, summed in 64 bits."""
+    st = synth.small_stack(230 + W, N, H, W, K=3, nan_frac=0.1, n_angles=5, n_speeds=5, s_hi=6.0, n_sources=1, flux=30.0)
+    s = _stack(kb, ctx, st, "f32")
+    job = kb.Job(ctx, H, W, N, st.vx.size, k)
+    job.search(s, st.times, st.vx, st.vy)
+    rec, got = job.results(), job.filter_lightcurves(s, 1e6)
+    y, x, _ = np.meshgrid(np.arange(H), np.arange(W), np.arange(k), indexing="ij")
+    assert np.array_equal(got["x0"], x) and np.array_equal(got["y0"], y) and np.array_equal(got["vidx"], rec["vidx"])
+    assert np.array_equal(got["nobs"], np.where(rec["vidx"] >= 0, rec["nobs"], 0)) and not got["nrejected"].any()
+    # N FP32 additions against FP64 ones: N roundings of the partial sums, each at most the sum of the sizes
+    planes = np.empty((N, H, W, 2), np.float32)
+    s.copy_planes(0, planes)
+    bound = N * 2.0 ** -24 * np.abs(planes).sum(0).max((0, 1)) * N
+    assert np.abs(got["psi"] - rec["psi"]).max() <= bound[0] and np.abs(got["phi"] - rec["phi"]).max() <= bound[1]
+    job.free()
+    s.free()
