@@ -122,3 +122,37 @@ def test_cluster_arguments_are_checked(kb, ctx):
     assert label.numel() == 0 and groups == 0
     # the context stays usable after the errors
     _compare(kb, ctx, rec, 1.0, 1.0, 1.0, 2)
+
+
+@pytest.mark.parametrize("ms", [1, 2, 3])
+def test_isolated_points_beside_groups(kb, ctx, ms):
+    """Points alone in their 81 cells, pairs just within and just beyond eps, and groups of five."""
+    rng = np.random.default_rng(ms)
+    n = 3000
+    rec = np.zeros(n, kb.RESULT_DTYPE)
+    cell = rng.permutation(n) // np.repeat([1, 2, 5], n // 3)   # of 1, 2 or 5 points
+    rec["x0"], rec["y0"] = 40 * (cell % 60), 40 * (cell // 60)
+    rec["x0"] += rng.integers(0, 4, n)
+    rec["vx"], rec["vidx"], rec["nu"] = rng.integers(0, 3, n), rng.integers(-1, 30, n), rng.normal(5.0, 1.0, n)
+    dev = torch.from_numpy(rec.view(np.uint8).copy()).to(DEV)
+    label, keep, core, groups = ctx.cluster(dev, 1.0, 1.0, 2.0, ms, core=True)
+    p = np.stack([rec["x0"], rec["y0"], rec["vx"], rec["vy"]], 1).astype(np.float32)
+    ok = rec["vidx"] >= 0
+    near = np.zeros((n, n), bool)
+    for i in range(n):
+        near[i] = (((p[i] - p) ** 2).sum(1) <= 4.0) & ok & ok[i]
+    want_core = ok & (near.sum(1) >= ms)
+    want = np.where(ok, np.arange(n), -1)
+    for _ in range(n):
+        new = want.copy()
+        for i in np.flatnonzero(want_core):
+            new[i] = want[near[i] & want_core].min()
+        if np.array_equal(new, want):
+            break
+        want = new
+    for i in np.flatnonzero(ok & ~want_core):
+        c = np.flatnonzero(near[i] & want_core)
+        if c.size:
+            want[i] = want[c[np.lexsort((c, ((p[i] - p[c]) ** 2).sum(1)))[0]]]
+    assert np.array_equal(core.cpu().numpy(), want_core) and np.array_equal(label.cpu().numpy(), want)
+    assert groups == np.unique(want[ok]).size == int(keep.sum())
