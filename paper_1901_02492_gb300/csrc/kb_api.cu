@@ -1551,9 +1551,9 @@ int kb_cluster(kb_ctx *ctx, const kb_result *cand, size_t n, const kb_cluster_pa
     cudaStream_t st = (cudaStream_t)stream;
     int T = 1;
     while (T < 2 * (int)n) T <<= 1;
-    const size_t words = 3 * (size_t)T + 5 * n;   // owner, cnt, start | slot, rank, run_idx, parent, bestidx
-    const size_t bytes = 3 * n * sizeof(int4) + n * sizeof(unsigned long long) + words * sizeof(int) +
-                         3 * sizeof(int) + 2 * n + 16;
+    const size_t words = (size_t)T + 5 * n;   // owner | cnt, start, run_idx, parent, bestidx
+    const size_t bytes = 2 * n * sizeof(int4) + n * sizeof(unsigned long long) + words * sizeof(int) +
+                         3 * sizeof(int) + 2 * n;
     void *buf = nullptr;
     size_t acct = 0;
     int rc = dev_alloc(ctx, bytes, &buf, &acct);
@@ -1576,18 +1576,17 @@ int kb_cluster(kb_ctx *ctx, const kb_result *cand, size_t n, const kb_cluster_pa
     a.eps2_lo = f32 ? (float)(a.eps2 * (1.0 - 0x1p-16)) : NAN;
     a.eps2_hi = f32 ? (float)(a.eps2 * (1.0 + 0x1p-16)) : NAN;
     a.min_samples = p->min_samples;
-    a.pts = reinterpret_cast<int4 *>(buf);
-    a.cells = a.pts + n;
+    a.cells = reinterpret_cast<int4 *>(buf);
     a.run_pts = a.cells + n;
     unsigned long long *bestnu = reinterpret_cast<unsigned long long *>(a.run_pts + n);
     int *w = reinterpret_cast<int *>(bestnu + n);
     a.bestnu = bestnu;
     a.owner = w;
     a.cnt = w + T;
-    a.start = w + 2 * (size_t)T;
-    a.slot = w + 3 * (size_t)T;
-    a.rank = a.slot + n;
-    a.run_idx = a.rank + n;
+    a.start = a.cnt + n;
+    a.run_idx = a.start + n;
+    a.first = reinterpret_cast<int *>(bestnu);
+    a.rank = a.first + n;
     a.parent = a.run_idx + n;
     a.bestidx = a.parent + n;
     a.count = reinterpret_cast<unsigned *>(a.bestidx + n);

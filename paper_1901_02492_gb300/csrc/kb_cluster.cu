@@ -89,18 +89,22 @@ __device__ __forceinline__ unsigned hash4(int4 c, unsigned mask) {
     return (unsigned)h & mask;
 }
 
+__device__ __forceinline__ int4 point_of(const kb_result &r) {
+    return make_int4(r.x0, r.y0, __float_as_int(r.vx), __float_as_int(r.vy));
+}
+
 __device__ __forceinline__ bool same_cell(const ClusterArgs &a, int o, int4 c) {
     const int4 d = a.cells[o];
     return d.x == c.x && d.y == c.y && d.z == c.z && d.w == c.w;
 }
 
-// Slot of cell c in the finished table, or -1.
-__device__ int find_slot(const ClusterArgs &a, int4 c) {
+// The first candidate of cell c, or -1.
+__device__ int find_cell(const ClusterArgs &a, int4 c) {
     unsigned s = hash4(c, a.T - 1);
     for (int probe = 0; probe < a.T; ++probe) {
         const int o = a.owner[s];
         if (o < 0) return -1;
-        if (same_cell(a, o, c)) return (int)s;
+        if (same_cell(a, o, c)) return o;
         s = (s + 1) & (a.T - 1);
     }
     return -1;
@@ -127,11 +131,10 @@ __global__ void init_kernel(ClusterArgs a) {
     const int stride = gridDim.x * blockDim.x;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.T; s += stride) {
         a.owner[s] = -1;
-        a.cnt[s] = 0;
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+        a.cnt[i] = 0;
         a.parent[i] = i;
-        a.bestnu[i] = 0ull;
         a.bestidx[i] = 0x7fffffff;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -150,7 +153,6 @@ __global__ void prep_kernel(ClusterArgs a) {
             atomicExch(a.status, 1);
             ok = false;
         }
-        a.pts[i] = make_int4(r.x0, r.y0, __float_as_int(r.vx), __float_as_int(r.vy));
         a.cells[i] = c;
         a.valid[i] = ok ? 1 : 0;
     }
@@ -165,22 +167,26 @@ __global__ void insert_kernel(ClusterArgs a) {
         for (int probe = 0; probe < a.T && !placed; ++probe) {
             const int o = atomicCAS(&a.owner[s], -1, i);
             if (o == -1 || same_cell(a, o, c)) {
-                a.slot[i] = (int)s;
-                a.rank[i] = atomicAdd(&a.cnt[s], 1);
+                const int first = o == -1 ? i : o;
+                a.first[i] = first;
+                a.rank[i] = atomicAdd(&a.cnt[first], 1);
                 placed = true;
             } else {
                 s = (s + 1) & (a.T - 1);
             }
         }
-        if (!placed) atomicExch(a.status, 2);
+        if (!placed) {   // no slot left: the point takes no part
+            atomicExch(a.status, 2);
+            a.valid[i] = 0;
+        }
     }
 }
 
-// the place of every occupied cell's run
+// the place of every cell's run
 __global__ void place_kernel(ClusterArgs a) {
     const int lane = threadIdx.x & 31;
-    for (int s0 = blockIdx.x * blockDim.x + threadIdx.x - lane; s0 < a.T; s0 += gridDim.x * blockDim.x) {
-        const int s = s0 + lane, c = s < a.T ? a.cnt[s] : 0;
+    for (int s0 = blockIdx.x * blockDim.x + threadIdx.x - lane; s0 < a.n; s0 += gridDim.x * blockDim.x) {
+        const int s = s0 + lane, c = s < a.n ? a.cnt[s] : 0;
         int end = c;   // one atomic for the warp's cells
 #pragma unroll
         for (int o = 1; o < 32; o *= 2) {
@@ -197,8 +203,8 @@ __global__ void place_kernel(ClusterArgs a) {
 __global__ void gather_kernel(ClusterArgs a) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
         if (!a.valid[i]) continue;
-        const int at = a.start[a.slot[i]] + a.rank[i];
-        a.run_pts[at] = a.pts[i];
+        const int at = a.start[a.first[i]] + a.rank[i];
+        a.run_pts[at] = point_of(a.cand[i]);
         a.run_idx[at] = i;
     }
 }
@@ -219,7 +225,7 @@ __device__ __forceinline__ bool for_neighbours(const ClusterArgs &a, int i, int 
         count = 0;
         start = 0;
         if (d < 81) {
-            const int s = find_slot(a, make_int4(c.x + d % 3 - 1, c.y + (d / 3) % 3 - 1, c.z + (d / 9) % 3 - 1, c.w + d / 27 - 1));
+            const int s = find_cell(a, make_int4(c.x + d % 3 - 1, c.y + (d / 3) % 3 - 1, c.z + (d / 9) % 3 - 1, c.w + d / 27 - 1));
             if (s >= 0) {
                 count = a.cnt[s];
                 start = a.start[s];
@@ -276,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 8) core_kernel(ClusterArgs a) {
         const bool ok = a.valid[i] != 0;
         int cnt = 0;
         if (ok) {
-            const int4 p = a.pts[i];
+            const int4 p = point_of(a.cand[i]);
             const bool near = for_neighbours<FIRST>(a, i, lane, [&](int at, bool on) {
                 cnt += __popc(__ballot_sync(0xffffffffu, on && within(a, p, a.run_pts[at])));
                 return cnt < a.min_samples;
@@ -286,7 +292,10 @@ __global__ void __launch_bounds__(kThreads, 8) core_kernel(ClusterArgs a) {
                 if (lane == 0) a.valid[i] = kAlone;
             }
         }
-        if (lane == 0) a.core[i] = (ok && cnt >= a.min_samples) ? 1 : 0;
+        if (lane == 0) {
+            a.core[i] = (ok && cnt >= a.min_samples) ? 1 : 0;
+            a.bestnu[i] = 0ull;
+        }
     }
 }
 
@@ -295,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 8) union_kernel(ClusterArgs a) {
     const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x / 32);
     for (int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < a.n; i += warps) {
         if (!a.core[i] || a.valid[i] == kAlone) continue;
-        const int4 p = a.pts[i];
+        const int4 p = point_of(a.cand[i]);
         for_neighbours<EACH>(a, i, lane, [&](int at, bool on) {
             const int j = on ? a.run_idx[at] : i;
             if (j < i && a.core[j]) {
@@ -331,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, 8) label_kernel(ClusterArgs a) {
             int best = i;
             if (!a.core[i] && a.valid[i] != kAlone) {
                 // the nearest core neighbour (smallest d2, then lowest index)
-                const int4 p = a.pts[i];
+                const int4 p = point_of(a.cand[i]);
                 int bj = 0x7fffffff;
                 double bd = INFINITY;
                 for_neighbours<ALL>(a, i, lane, [&](int at, bool on) {
@@ -396,7 +405,7 @@ cudaError_t launch_cluster(const ClusterArgs &a, int sm_count, cudaStream_t st) 
     if (a.n > 0) {
         prep_kernel<<<grid(a.n), kThreads, 0, st>>>(a);
         insert_kernel<<<grid(a.n), kThreads, 0, st>>>(a);
-        place_kernel<<<grid(a.T), kThreads, 0, st>>>(a);
+        place_kernel<<<grid(a.n), kThreads, 0, st>>>(a);
         gather_kernel<<<grid(a.n), kThreads, 0, st>>>(a);
         core_kernel<<<grid(32LL * a.n), kThreads, 0, st>>>(a);
         union_kernel<<<grid(32LL * a.n), kThreads, 0, st>>>(a);

@@ -379,11 +379,13 @@ struct ClusterArgs {
     double w_pos, w_vel, eps2, inv_side;
     int min_samples;
     float eps2_lo, eps2_hi;  // FP32 distances below / above these are decided (NaN: none is)
-    int4 *pts, *cells;       // [n] packed (x0, y0, vx bits, vy bits), grid cell
-    int4 *run_pts;           // [n] the points, cell by cell
+    int4 *cells;             // [n] grid cell
+    int4 *run_pts;           // [n] the points, packed (x0, y0, vx bits, vy bits), cell by cell
     uint8_t *valid;          // [n] takes part (vidx >= 0, cell in range)
-    int *owner, *cnt, *start;  // [T] first candidate of the slot's cell, its points, their run in run_pts
-    int *slot, *rank;        // [n] the point's slot and its place in the run
+    int *owner;              // [T] first candidate of the slot's cell, which stands for the cell below
+    int *cnt, *start;        // [n] a cell's points, their run in run_pts
+    int *first, *rank;       // [n] the point's cell and its place in the run; the same memory as bestnu,
+                             // which is set once the runs are filled
     int *run_idx;            // [n] candidate of run_pts
     int *parent;             // [n]
     int *cursor;             // places given out

@@ -156,3 +156,18 @@ def test_isolated_points_beside_groups(kb, ctx, ms):
             want[i] = want[c[np.lexsort((c, ((p[i] - p[c]) ** 2).sum(1)))[0]]]
     assert np.array_equal(core.cpu().numpy(), want_core) and np.array_equal(label.cpu().numpy(), want)
     assert groups == np.unique(want[ok]).size == int(keep.sum())
+
+
+@pytest.mark.parametrize("n", [1, 700, 1024, 1025])
+def test_scratch_within_the_linked_lists_size(kb, n):
+    """The scratch of a call stays within 54 bytes per candidate, 8 per hash slot (2 n of them, rounded up to
+    a power of two) and 24: a budget of that much is enough."""
+    slots = 1
+    while slots < 2 * n:
+        slots *= 2
+    c = kb.Context(0, 54 * n + 8 * slots + 24)
+    rec = np.zeros(n, kb.RESULT_DTYPE)
+    rec["x0"], rec["nu"] = np.arange(n), np.arange(n)
+    label, keep, _, groups = c.cluster(torch.from_numpy(rec.view(np.uint8).copy()).to(DEV), 1.0, 1.0, 1.5, 2)
+    assert groups == 1 and int(keep[n - 1]) == 1 and not label.any()
+    c.close()
