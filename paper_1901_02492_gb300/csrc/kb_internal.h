@@ -238,6 +238,17 @@ inline bool search_idx32(const SearchArgs &a, bool elements) {
     if (elements || a.k > kShortMax) return a.planes_elems < (1LL << 31) - 1;
     return a.planes_elems * (a.storage == KB_F32 ? (long long)sizeof(float2) : (long long)sizeof(pair16)) < (1LL << 32);
 }
+// Lets launches of `kern` take all the dynamic shared memory a CTA can have.  Function attributes
+// belong to the device's context, not to a kb_ctx: threads with contexts of their own launch the same
+// kernels side by side, so the limit is one value whatever a launch needs.  Set to each launch's own
+// size, another thread's smaller one in between made a launch fail.
+template <class K>
+cudaError_t allow_smem(K *kern) {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)fa.sharedSizeBytes);
+}
 // register-gather kernel (variant 0 = its default shape, 1..4)
 cudaError_t launch_search(const SearchArgs &a, cudaStream_t st);
 // one storage's kernels (kb_search.cu, kb_search_bf16.cu, kb_search_f16.cu)

@@ -85,24 +85,19 @@ __global__ void __launch_bounds__(kThreads) snr2_kernel(SnrArgs a) {
 cudaError_t launch_snr2(const SnrArgs &a, cudaStream_t st) {
     if (a.span % 32 != 0) return cudaErrorInvalidValue;
     const dim3 grid(a.H, a.N);
-    const size_t smem = (size_t)((a.W + 31) / 32) * sizeof(float);
-    cudaError_t e;
+    const size_t smem = (size_t)((a.W + 31) / 32) * sizeof(float);   // at most 4 KB
     switch (a.storage) {
         case KB_F32:
-            e = cudaFuncSetAttribute(snr2_kernel<KB_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess) snr2_kernel<KB_F32><<<grid, kThreads, smem, st>>>(a);
+            snr2_kernel<KB_F32><<<grid, kThreads, smem, st>>>(a);
             break;
         case KB_BF16:
-            e = cudaFuncSetAttribute(snr2_kernel<KB_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess) snr2_kernel<KB_BF16><<<grid, kThreads, smem, st>>>(a);
+            snr2_kernel<KB_BF16><<<grid, kThreads, smem, st>>>(a);
             break;
         case KB_F16:
-            e = cudaFuncSetAttribute(snr2_kernel<KB_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess) snr2_kernel<KB_F16><<<grid, kThreads, smem, st>>>(a);
+            snr2_kernel<KB_F16><<<grid, kThreads, smem, st>>>(a);
             break;
         default: return cudaErrorInvalidValue;
     }
-    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

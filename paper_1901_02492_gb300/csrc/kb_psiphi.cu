@@ -602,8 +602,7 @@ static size_t psi_phi_smem(int K, bool sep) {
 
 template <int KT>
 cudaError_t launch_sep(const PsiPhiArgs &a, dim3 grid, size_t smem, cudaStream_t st) {
-    cudaError_t err = cudaFuncSetAttribute(psi_phi_sep_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+    cudaError_t err = allow_smem(psi_phi_sep_kernel<KT>);
     if (err != cudaSuccess) return err;
     psi_phi_sep_kernel<KT><<<grid, THREADS, smem, st>>>(a);
     return cudaGetLastError();
@@ -614,8 +613,7 @@ cudaError_t launch_gen(const PsiPhiArgs &a, dim3, size_t, cudaStream_t st) {
     constexpr int r = KT / 2;
     const dim3 grid((a.W + TX - 1) / TX, (a.H + GTY - 1) / GTY, a.N);
     const size_t smem = ((2 * KT * KT + 3) & ~3) * sizeof(float) + (size_t)(GTY + 2 * r) * (TX + 2 * r) * sizeof(float2);
-    cudaError_t err = cudaFuncSetAttribute(psi_phi_gen_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+    cudaError_t err = allow_smem(psi_phi_gen_kernel<KT>);
     if (err != cudaSuccess) return err;
     psi_phi_gen_kernel<KT><<<grid, THREADS, smem, st>>>(a);
     return cudaGetLastError();
@@ -635,8 +633,7 @@ cudaError_t launch_stream(const PsiPhiArgs &a0, cudaStream_t st) {
     while (a.seg > SY && strips * ((a.H + a.seg - 1) / a.seg) < 152 * 3) a.seg = (a.seg / 2 + SY - 1) / SY * SY;
     const dim3 grid((a.W + TX - 1) / TX, (a.H + a.seg - 1) / a.seg, a.N);
     const size_t smem = G::taps_bytes + G::raw_bytes + G::a_bytes + G::ring_bytes + (a.mask ? G::mask_bytes : 0);
-    cudaError_t err = cudaFuncSetAttribute(psi_phi_stream_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+    cudaError_t err = allow_smem(psi_phi_stream_kernel<KT>);
     if (err != cudaSuccess) return err;
     psi_phi_stream_kernel<KT><<<grid, THREADS, smem, st>>>(a);
     return cudaGetLastError();
@@ -695,7 +692,7 @@ cudaError_t launch_psi_phi(const PsiPhiArgs &a, cudaStream_t st) {
         case 21: return launch_gen<21>(a, grid, smem, st);
         default: break;
     }
-    cudaError_t err = cudaFuncSetAttribute(psi_phi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_smem(psi_phi_kernel);
     if (err != cudaSuccess) return err;
     psi_phi_kernel<<<grid, THREADS, smem, st>>>(a);
     return cudaGetLastError();

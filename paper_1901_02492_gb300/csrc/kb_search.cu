@@ -1043,11 +1043,11 @@ cudaError_t launch_pt(const SearchArgs &search, cudaStream_t st) {
         }
     }
     a.slots = a.k + cap;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // Shared-memory carveout: the driver's choice unless the caller sets one
+    err = allow_smem(kern);
+    // Shared-memory carveout: the driver's choice (-1) unless the caller sets one
     // (kb_set_search_carveout); it trades resident CTAs against the L1 that the
     // early epochs' gathers reuse across velocities.
-    if (err == cudaSuccess && a.carveout >= 0)
+    if (err == cudaSuccess)
         err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, a.carveout);
     if (err != cudaSuccess) return err;
     if (parts > 1) {
@@ -1149,8 +1149,8 @@ cudaError_t launch_batch_pt(const SearchArgs *jobs, const int4 *items, int n_ite
         if (cap < CAP) kern = search_batch_kernel<STORAGE, P, C, KM, I, true>;
     }
     const size_t smem = tile_smem<STORAGE, P, KM, I>(kmax, cap);
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err == cudaSuccess && carve >= 0)
+    err = allow_smem(kern);
+    if (err == cudaSuccess)
         err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
     int per_sm = 0;
     if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, smem);

@@ -326,8 +326,7 @@ cudaError_t launch_tma(const SearchArgs &a, cudaStream_t st) {
                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     const TmaLayout L = tma_layout(S, Tl::SLOT, a.N, a.k, P);
-    cudaError_t err = cudaFuncSetAttribute(search_tma_kernel<STORAGE, P, S, C>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+    cudaError_t err = allow_smem(search_tma_kernel<STORAGE, P, S, C>);
     if (err != cudaSuccess) return err;
     dim3 grid((a.W + 32 * P - 1) / (32 * P), (a.H + CWARPS - 1) / CWARPS);
     search_tma_kernel<STORAGE, P, S, C><<<grid, TTHREADS, L.total, st>>>(map, a);
