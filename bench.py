@@ -223,15 +223,6 @@ def measured_peaks():
         return {}
 
 
-def search_span(storage, variant, k):
-    """Pixels per warp span of the register-gather search shape (the library's search_span)."""
-    p32, p16 = [2, 4, 2, 4, 2], [2, 2, 1, 2, 1]
-    v = variant if 1 <= variant <= 4 else 0
-    if storage != "f32" and v == 0 and k > 8:
-        return 64
-    return 32 * p32[v] if storage == "f32" else 64 * p16[v]
-
-
 def psf_moment_cuts(psf, aperture):
     """Moment-filter cuts from the epochs' PSFs: each PSF's per-axis second moment s^2 (of the
     sampled kernel), the second moment of that Gaussian inside the aperture, s^2 (1 - u e^-u /
@@ -295,8 +286,8 @@ def search_byte_classes(binding, times, vx, vy, H, W, bytes_per_eval, span):
     comes from, counted on the host from the library's own offset table:
       ref      epochs at the reference time (offset 0 for every velocity): loaded once
                per start pixel, then reused for every velocity;
-      off      trajectory pixel outside the image: nothing to gather (the kernel reads
-               a zero block that stays in L1);
+      off      trajectory pixel outside the image: nothing to gather (epochs that take a
+               whole tile off the image are left out of its table);
       gathered trajectory pixel inside the image: one pair gathered per evaluation.
     Algorithmic bytes per launch = gathered evaluations + one load per pixel and
     reference epoch, times the pair size.  `issued` counts what the kernel loads: whole
@@ -424,9 +415,9 @@ def run_ours(args):
     var = var_h.to(dev)
     stream = torch.cuda.current_stream(dev)
     # roofline denominators, before the timed region: the L2-to-SM rate of the search's own
-    # access form (the warp span of the launch shape, 512 B for the default shapes, at any 8-byte offset),
+    # access form (the warp span of the launch shape, at any 8-byte offset),
     # and of line-aligned spans for reference
-    span = search_span(args.storage, args.variant, job_kkeep(k, args.rescore, args.storage))
+    span = kb.search_span(args.storage, args.variant, V, k, flags)
     span_bytes = span * BYTES_PER_EVAL[args.storage]
     gather_peak = ctx.measure_gather_peak(span_bytes, 8)
     gather_peak_aligned = ctx.measure_gather_peak(span_bytes, 256)

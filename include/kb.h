@@ -111,9 +111,8 @@ size_t kb_hbm_in_use(const kb_ctx *ctx);
  * first one since the last reset is recorded, never trapped.
  * kb_debug_build: 1 in a KB_DEBUG build, 0 otherwise.
  * kb_debug_word: *word = (site << 56) | offset of that first access (0 if none;
- * sites: 1 reference-epoch gather, 2 batched gather, 3 remainder gather,
- * 4 predicated gather, byte offsets from the planes' base; 5 table entry,
- * 6 list column, element indices); reset != 0 clears it afterwards.  It
+ * sites: 1 reference-epoch gather, 2 batched gather, 3 remainder gather, byte
+ * offsets from the planes' base; 5 table entry, 6 list column, element indices); reset != 0 clears it afterwards.  It
  * synchronises the device.  KB_EINVAL in a build without KB_DEBUG or for a
  * NULL argument. */
 int kb_debug_build(void);
@@ -155,6 +154,12 @@ int kb_set_search_swizzle(kb_ctx *ctx, int cols);
  * 12 x 4096^2 stack: 97.7, 102.5 and 98.7 ms.  Ties in nu are broken by the
  * caller's velocity index, so results do not depend on it. */
 int kb_set_search_order(kb_ctx *ctx, int order);
+
+/* The start pixels of one warp row of kb_search with these arguments (the width of its tiles): the
+ * span of consecutive pixels, 8 bytes each in FP32 and 4 in 16-bit storage, that a warp reads for one
+ * velocity and epoch.  variant as for kb_set_search_variant, the others as for kb_search (KB_PRUNE:
+ * with nu_min > 0).  0 for arguments that kb_search would reject.  Pure host function. */
+int kb_search_span(int storage, int variant, int V, int topk, int flags);
 
 /* Measurement helper (no counterpart in the paper): the L2-to-SM bandwidth, in
  * GB/s, of the search's own access form -- each warp reads warp_bytes (256, 512

@@ -86,6 +86,7 @@ _kb_job_repaired = _sig("kb_job_repaired", _i32, [_P, ctypes.POINTER(_sz)])
 _kb_make_psi_phi_static = _sig("kb_make_psi_phi_static", _i32,
                                [_P, _P, _P, _P, _i32, _i32, _i32, _i32, _f32, _P, _P])
 
+_kb_search_span = _sig("kb_search_span", _i32, [_i32, _i32, _i32, _i32, _i32])
 _kb_estimate_bytes = _sig("kb_estimate_bytes", _i32, [_i32, _i32, _i32, _i32, _i32, _i32, _i32, _i32,
                                                        ctypes.POINTER(_sz), ctypes.POINTER(_sz)])
 _kb_filter_lightcurves = _sig("kb_filter_lightcurves", _i32, [_P, _P, ctypes.c_double, _P, _sz, ctypes.POINTER(_sz), _P])
@@ -334,6 +335,15 @@ def estimate_bytes(N, H, W, storage, K, V, topk, flags=0):
     if rc != KB_OK:
         raise KBError(rc, "kb_estimate_bytes rejected the shape")
     return int(a.value), int(b.value)
+
+
+def search_span(storage, variant, V, topk, flags=0):
+    """Start pixels of one warp row of a search with these arguments (kb_search_span)."""
+    st = STORAGE[storage] if isinstance(storage, str) else int(storage)
+    span = _kb_search_span(st, int(variant), int(V), int(topk), int(flags))
+    if span <= 0:
+        raise KBError(KB_EINVAL, "kb_search_span rejected the arguments")
+    return span
 
 
 def offsets(times, vx, vy):

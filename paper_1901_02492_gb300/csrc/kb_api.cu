@@ -604,6 +604,17 @@ int kb_estimate_bytes(int N, int H, int W, int storage, int K, int V, int topk, 
     return KB_OK;
 }
 
+int kb_search_span(int storage, int variant, int V, int topk, int flags) {
+    if ((storage != KB_F32 && storage != KB_BF16 && storage != KB_F16) || variant < 0 || variant > 8 || V < 1 ||
+        V > KB_MAX_VELOCITIES || topk < 1 || topk > KB_MAX_TOPK || (flags & ~(KB_RESCORE_FP64 | KB_PRUNE)))
+        return 0;
+    if (variant >= 5) return variant <= 6 ? 64 : 128;   // the pipelined kernel's 2 or 4 pixels per lane
+    const int k = job_kkeep(topk, flags, storage);
+    const bool pruned = variant == 0 && (flags & KB_PRUNE);
+    const bool keys = variant == 0 && !pruned && (flags & KB_RESCORE_FP64) && kb::search_key_lists(V, k);
+    return kb::search_span(storage, kb::search_shape(storage, variant, k, keys, pruned));
+}
+
 int kb_job_create(kb_ctx *ctx, int H, int W, int N, int V, int topk, int flags, kb_job **out) {
     if (!ctx || !out) return KB_EINVAL;
     *out = nullptr;
@@ -906,7 +917,7 @@ int kb_search(kb_job *job, const kb_stack *s, const double *times, const double 
     // after every kb_make_psi_phi) on this stream; only a positive nu_min can prune
     if ((flags & KB_PRUNE) && nu_min > 0.0f && a.variant == 0) {
         kb_stack *ms = const_cast<kb_stack *>(s);   // the bound planes are a cache of the stack
-        const int span = kb::search_auto_span(a.storage, a.k);
+        const int span = kb::search_span(a.storage, kb::search_shape(a.storage, 0, a.k, false, true));
         const size_t need = (size_t)ms->N * ms->H * ((ms->W + 31) / 32 + span / 32) * sizeof(float);
         if (ms->snr2 && ms->snr2_bytes != need) {
             cudaStreamWaitEvent(ctx->astream, ms->used, 0);
@@ -1005,7 +1016,7 @@ int index_bits(const kb::SearchArgs &a) { return kb::search_idx32(a, false) ? 32
 // about `frac` of each search's rows from its middle.
 void make_items(const kb_batch *b, int g, int variant, double frac, std::vector<int4> &out) {
     out.clear();
-    const int span = kb::search_span(b->groups[g].storage, variant, b->groups[g].kmax), R = kb::kTileRows;
+    const int span = kb::search_span(b->groups[g].storage, variant), R = kb::kTileRows;
     for (int j : b->group_jobs[g]) {
         const kb::SearchArgs &a = b->args[j];
         const int tx = (a.W + span - 1) / span, ty = (a.H + R - 1) / R;
@@ -1132,7 +1143,7 @@ int kb_batch_create(kb_ctx *ctx, int count, const kb_batch_item *items, int flag
             memset(&G, 0, sizeof G);
             G.storage = a.storage;
             G.index_bits = bits;
-            G.variant = kb::default_variant(a.storage, a.k);
+            G.variant = kb::search_shape(a.storage, 0, a.k, false, false);
             G.kmax = a.k;
             b->groups.push_back(G);
             b->group_jobs.emplace_back();

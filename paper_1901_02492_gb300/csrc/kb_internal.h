@@ -288,8 +288,6 @@ cudaError_t debug_word(unsigned long long *word, bool reset);
 // the FP64 rescoring): the records' nu are then rounded upwards to 32 - key_bits bits
 // of their order-preserving FP32 encoding
 bool search_keys(const SearchArgs &a);
-// the automatic shape's span for lists of k (pixels per warp, the KB_PRUNE window)
-int search_auto_span(int storage, int k);
 
 // likelihood bound planes of the thresholded search (kb_prune.cu)
 struct SnrArgs {
@@ -308,10 +306,13 @@ cudaError_t launch_search_tma(const SearchArgs &a, cudaStream_t st);
 // carve = shared-memory carveout percent (-1: the automatic rule)
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
                                 int variant, int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st);
-// pixels per CTA row segment of a register-gather shape (tile width) for lists of k
-int search_span(int storage, int variant, int k);
-// the explicit shape (1..4) that the automatic choice (variant 0) takes for lists of k
-int default_variant(int storage, int k);
+// the explicit shape (1..4) that a search with lists of k takes: `variant` itself, or for 0 the
+// automatic choice, which key lists and pruned searches have their own of
+int search_shape(int storage, int variant, int k, bool keys, bool pruned);
+// pixels per CTA row segment (tile width) of an explicit shape
+int search_span(int storage, int shape);
+// whether a rescoring search of V velocities keeps its k candidates as keys (unless pruned)
+bool search_key_lists(int V, int k);
 // rows per CTA tile of the register-gather kernel
 constexpr int kTileRows = 8;
 

@@ -849,12 +849,14 @@ __device__ __forceinline__ void search_tile(const SearchArgs &a, int bx, int by,
 
 // Resident CTAs per SM the register allocation is held to, by shape.  Lists up to 8
 // long: the narrow shapes (FP32 with two pixels per lane, 16-bit with one pixel pair) are
-// held to 4 CTAs (64 registers: the loop keeps everything in registers; at 5 CTAs, 48
-// registers, it spills in the loop: 12 x 4096^2, k = 8, 136 ms against 76); 16-bit with
-// two pixel pairs per lane to 3 with 4-epoch batches (80 registers) and 2 with 8-epoch
-// batches.  Longer lists: 3.  The wide FP32 shapes: 2.  The batch kernel, which keeps its
-// search's arguments in shared memory rather than the parameter bank and so needs more
-// registers, is held to 3 for the narrow shapes and 2 for the others.
+// held to 4 CTAs (64 registers; at 5 CTAs, 48 registers, FP32 spills in the loop: 12 x 4096^2,
+// k = 8, 136 ms against 76); 16-bit with two pixel pairs per lane to 3 with 4-epoch batches
+// (80 registers) and 2 with 8-epoch batches.  Longer lists: 3.  The wide FP32 shapes: 2.  The
+// batch kernel, which keeps its search's arguments in shared memory rather than the parameter
+// bank and so needs more registers, is held to 3 for the narrow shapes and 2 for the others.
+// FP32's automatic kernels and FP16's value lists fit; a few values of the others live in local
+// memory: BF16 (1, 4) 8 bytes of stores, key lists (2, 4) 16, BF16 (1, 8) with lists of 9 to 16 52,
+// BF16's batch kernels 4 to 52, pruned FP32 with lists up to 8 8 (its form for many epochs none).
 template <int STORAGE, int P, int C, int KM, bool KEYS>
 constexpr int min_ctas() {
     constexpr bool narrow = STORAGE == KB_F32 ? P <= 2 : P <= 1;
@@ -1086,9 +1088,8 @@ cudaError_t launch_keys(const SearchArgs &a, cudaStream_t st) {
 }
 
 // key form where it keeps at least 11 of nu's 23 fraction bits (up to 4096 velocities)
-bool use_keys(const SearchArgs &a) {
-    return a.cand_only && !a.snr2 && a.k <= kKeyMax && a.key_bits >= 1 && a.key_bits <= 12;
-}
+bool key_lists(int V, int k) { return k <= kKeyMax && V <= 4096; }
+bool use_keys(const SearchArgs &a) { return a.cand_only && !a.snr2 && key_lists(a.V, a.k); }
 
 // 32-bit offsets when every plane of both phases (and the bound planes) is in their reach
 template <int STORAGE, int P, int C, bool PRUNE = false>
@@ -1099,37 +1100,33 @@ cudaError_t launch_idx(const SearchArgs &a, cudaStream_t st) {
     return launch_one<STORAGE, P, C, long long, PRUNE>(a, st);
 }
 
-// Shapes: (loads per lane P, epochs per load batch C); a 16-bit load is two pixels.
-// Defaults (variant 0): FP32 (2, 8), 12 x 4096^2, k = 8: 76 ms; 16-bit value lists up to 8
-// long (1, 4), 12 x 2048^2, 1024 velocities, k = 8, BF16 / FP16: 18.6 / 18.8 ms, (1, 8) 20.8 /
-// 20.7; longer ones (1, 8), 12 x 1800^2, 1024 velocities, k = 12, BF16: 18.7 ms, (1, 4) 21.9,
-// (2, 4) 20.8, (2, 8) 23.2.
+// Shapes: (loads per lane P, epochs per load batch C); a 16-bit load is two pixels.  search_shape
+// makes the choice.  Automatic: FP32 (2, 8), 12 x 4096^2, k = 8: 76 ms; 16-bit value lists up to 8
+// long (1, 4), 12 x 2048^2, 1024 velocities, k = 8, BF16 / FP16: 18.6 / 18.8 ms, (1, 8) 20.8 / 20.7;
+// longer ones (1, 8), 12 x 1800^2, 1024 velocities, k = 12, BF16: 18.7 ms, (1, 4) 21.9, (2, 4) 20.8,
+// (2, 8) 23.2.  Key lists take two pairs per lane, value lists one, whose merges fit the registers
+// beside the loop (pruned short ones two, as their bound planes' span has it).
 template <int STORAGE>
 cudaError_t launch_storage(const SearchArgs &a, cudaStream_t st) {
+    const bool own = a.variant == 0, keys = own && use_keys(a), pruned = own && a.snr2;
+    const int shape = search_shape(a.storage, a.variant, a.k, keys, pruned);
     if constexpr (STORAGE == KB_F32) {
-        switch (a.variant) {
+        if (pruned) return launch_idx<STORAGE, 2, 8, true>(a, st);
+        if (keys) return launch_keys<STORAGE, 2, 8>(a, st);
+        switch (shape) {
             case 1: return launch_idx<STORAGE, 4, 4>(a, st);
             case 2: return launch_idx<STORAGE, 2, 4>(a, st);
             case 3: return launch_idx<STORAGE, 4, 8>(a, st);
-            default:
-                if (a.snr2) return launch_idx<STORAGE, 2, 8, true>(a, st);
-                if (use_keys(a)) return launch_keys<STORAGE, 2, 8>(a, st);
-                return launch_idx<STORAGE, 2, 8>(a, st);
+            default: return launch_idx<STORAGE, 2, 8>(a, st);
         }
     } else {
-        switch (a.variant) {
+        if (pruned) return shape == 2 ? launch_idx<STORAGE, 1, 4, true>(a, st) : launch_idx<STORAGE, 2, 4, true>(a, st);
+        if (keys) return launch_keys<STORAGE, 2, 4>(a, st);
+        switch (shape) {
+            case 1: return launch_idx<STORAGE, 2, 4>(a, st);
             case 2: return launch_idx<STORAGE, 1, 4>(a, st);
             case 3: return launch_idx<STORAGE, 2, 8>(a, st);
-            case 4: return launch_idx<STORAGE, 1, 8>(a, st);
-            case 1: return launch_idx<STORAGE, 2, 4>(a, st);
-            // automatic: key lists take two pairs per lane; value lists one pair, whose merges
-            // fit the registers beside the loop (and pruned short ones two, as their bound
-            // planes' span has it)
-            default:
-                if (use_keys(a)) return launch_keys<STORAGE, 2, 4>(a, st);
-                if (a.snr2)
-                    return a.k > kShortMax ? launch_idx<STORAGE, 1, 4, true>(a, st) : launch_idx<STORAGE, 2, 4, true>(a, st);
-                return a.k > kShortMax ? launch_idx<STORAGE, 1, 8>(a, st) : launch_idx<STORAGE, 1, 4>(a, st);
+            default: return launch_idx<STORAGE, 1, 8>(a, st);
         }
     }
 }
@@ -1239,17 +1236,21 @@ cudaError_t debug_word(unsigned long long *word, bool reset) {
     return e;
 }
 
-int search_span(int storage, int variant, int k) {
-    // loads per lane P of the shape, times 32 lanes, times pixels per load
-    static const int p32[5] = {2, 4, 2, 4, 2}, p16[5] = {2, 2, 1, 2, 1};
-    const int v = (variant >= 1 && variant <= 4) ? variant : 0;
-    if (storage != KB_F32 && v == 0 && k > kShortMax) return 64;
-    return storage == KB_F32 ? 32 * p32[v] : 64 * p16[v];
+int search_shape(int storage, int variant, int k, bool keys, bool pruned) {
+    if (variant >= 1 && variant <= 4) return variant;
+    if (storage == KB_F32) return 4;                  // (2, 8)
+    if (keys) return 1;                               // (2, 4)
+    if (pruned) return k > kShortMax ? 2 : 1;         // (1, 4), (2, 4)
+    return k > kShortMax ? 4 : 2;                     // (1, 8), (1, 4)
 }
 
-int search_auto_span(int storage, int k) { return search_span(storage, 0, k); }   // of the pruned search
+int search_span(int storage, int shape) {
+    // loads per lane P of the shape, times 32 lanes, times pixels per load
+    static const int p32[5] = {0, 4, 2, 4, 2}, p16[5] = {0, 2, 1, 2, 1};
+    return storage == KB_F32 ? 32 * p32[shape] : 64 * p16[shape];
+}
 
-int default_variant(int storage, int k) { return storage != KB_F32 && k <= kShortMax ? 2 : 4; }   // (1, 4); (2, 8), (1, 8)
+bool search_key_lists(int V, int k) { return key_lists(V, k); }
 
 cudaError_t launch_search_batch(const SearchArgs *jobs, const int4 *items, int n_items, int *counter, int storage,
                                 int variant, int kmax, int njs, int carve, bool idx64, int sm_count, cudaStream_t st) {
