@@ -535,14 +535,15 @@ __device__ __forceinline__ double f64_of(float x) {
 // whether the FP64 test could reject the epoch (pe, fe): false only when it certainly does not.
 // With Pf, Ff the sums rounded to FP32 (relative error 2^-24), each product below is within
 // 2^-22 of its exact value, dev within 2^-21 (|pe Ff| + |Pf fe|) of its own and rest within
-// 2^-22 Ff; the comparison keeps another 2^-18.  Products that overflow or come near the
-// subnormal range are not judged here.
-__device__ __forceinline__ bool maybe_outlier(float pe, float fe, float Pf, float Ff, float ns2) {
+// 2^-22 Ff; the comparison keeps another 2^-18.  m is ns2 Ff, 0 where either is near the subnormal
+// range, as a subnormal factor of the right side would carry a larger error; products that overflow
+// or come near that range are not judged here.
+__device__ __forceinline__ bool maybe_outlier(float pe, float fe, float Pf, float Ff, float m) {
     const float a = pe * Ff, b = Pf * fe;
     const float dev = fabsf(a - b) + 0x1p-21f * (fabsf(a) + fabsf(b));
     const float rest = (Ff - fe) - 0x1p-22f * Ff;
-    const float right = ns2 * Ff * fe * rest;
-    return !(right > 1e-30f && right < 1e38f && dev * dev * (1.0f + 0x1p-18f) < right);
+    const float mf = m * fe, right = mf * rest;
+    return !(mf > 1e-30f && right > 1e-30f && right < 1e38f && dev * dev * (1.0f + 0x1p-18f) < right);
 }
 
 // NR: epochs whose values stay in registers between the passes (N <= NR), 0: gathered again
@@ -609,16 +610,17 @@ __global__ void __launch_bounds__(kFilterThreads) filter_kernel(FilterArgs a) {
             }
         }
         const float Pf = __double2float_rn(P), Ff = __double2float_rn(F), ns2 = (float)a.nsigma2;
+        const float m = ns2 > 1e-30f && ns2 * Ff > 1e-30f ? ns2 * Ff : 0.0f;
         bool maybe = false;
         if constexpr (NR > 0) {
 #pragma unroll
             for (int j = 0; j < NR; ++j)
-                if ((inside >> j & 1u) && q[j].y > 0.0f) maybe |= maybe_outlier(q[j].x, q[j].y, Pf, Ff, ns2);
+                if ((inside >> j & 1u) && q[j].y > 0.0f) maybe |= maybe_outlier(q[j].x, q[j].y, Pf, Ff, m);
         } else {
             for (int j = 0; j < a.N && !maybe; ++j) {
                 bool in;
                 const float2 w = value(j, in);
-                maybe = in && w.y > 0.0f && maybe_outlier(w.x, w.y, Pf, Ff, ns2);
+                maybe = in && w.y > 0.0f && maybe_outlier(w.x, w.y, Pf, Ff, m);
             }
         }
         Pk = P;

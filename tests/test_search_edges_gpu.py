@@ -262,3 +262,29 @@ def test_filter_on_strips_of_any_width(kb, ctx, N, H, W, k):
     assert np.abs(got["psi"] - rec["psi"]).max() <= bound[0] and np.abs(got["phi"] - rec["phi"]).max() <= bound[1]
     job.free()
     s.free()
+
+
+def test_filter_where_products_are_subnormal(kb, ctx):
+    """Two epochs whose phi lie 40 decades apart: the test's FP32 form has subnormal products on the way, and
+    must leave them to FP64.  Values within 2e-4 of the rejection limit, decided as the direct sums decide."""
+    rng = np.random.default_rng(5)
+    H, W, nsigma = 64, 64, 1e-10
+    phi = np.stack([10.0 ** rng.uniform(-36, -31, (H, W)), 10.0 ** rng.uniform(10, 14, (H, W))])
+    var = (1.0 / phi).astype(np.float32)
+    # |psi_0| F = nsigma sqrt(F phi_0 (F - phi_0)) up to 2e-4, psi_1 = 0
+    psi0 = nsigma * np.sqrt(phi[0]) * (1.0 + rng.uniform(-2e-4, 2e-4, (H, W)))
+    sci = np.stack([psi0 * var[0], np.zeros((H, W))]).astype(np.float32)
+    s = kb.Stack(ctx, 2, H, W, "f32")
+    s.make_psi_phi(torch.from_numpy(sci).to(DEV), torch.from_numpy(var).to(DEV), None, np.ones((2, 1, 1), np.float32))
+    job = kb.Job(ctx, H, W, 2, 1, 1)
+    job.search(s, np.array([0.0, 1.0]), np.zeros(1), np.zeros(1))
+    got = job.filter_lightcurves(s, nsigma)[..., 0]
+    p = np.empty((2, H, W, 2), np.float32)
+    s.copy_planes(0, p)
+    pe, fe = p[..., 0].astype(np.float64), p[..., 1].astype(np.float64)
+    P, F = pe[0] + pe[1], fe[0] + fe[1]
+    rest = F - fe
+    out = (fe > 0) & (rest > 0) & ((pe * F - P * fe) ** 2 > nsigma * nsigma * F * fe * rest)
+    assert np.array_equal(got["rejected"][..., 0], (out[0] + 2 * out[1]).astype(np.uint32)) and out.any() and not out.all()
+    job.free()
+    s.free()
