@@ -288,3 +288,41 @@ def test_filter_where_products_are_subnormal(kb, ctx):
     assert np.array_equal(got["rejected"][..., 0], (out[0] + 2 * out[1]).astype(np.uint32)) and out.any() and not out.all()
     job.free()
     s.free()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("N,H,W,V,k,s_hi", SHAPES)
+def test_every_shape_equals_the_pipelined_kernel(kb, ctx, storage, N, H, W, V, k, s_hi):
+    """The explicit shapes, which never share a tile's velocities between CTAs: several chunks of the table and
+    full buffers in the plain kernel (FP32's fourth shape is the automatic one, 16-bit's second and fourth are)."""
+    st = synth.small_stack(7 * N + k, N, H, W, K=5, nan_frac=0.05, n_angles=10, n_speeds=13, s_hi=s_hi, n_sources=3,
+                           flux=40.0)
+    s = _stack(kb, ctx, st, storage)
+    ctx.set_search_variant(5)
+    ref = _records(kb, ctx, s, st, V, k).tobytes()
+    for variant in (1, 2, 3, 4):
+        ctx.set_search_variant(variant)
+        assert _records(kb, ctx, s, st, V, k).tobytes() == ref, variant
+    ctx.set_search_variant(0)
+    s.free()
+
+
+@pytest.mark.parametrize("storage,k,flags", [("f32", 4, 0), ("f32", 12, 0), ("bf16", 8, 0), ("f16", 11, 0), ("bf16", 8, 1),
+                                             ("f16", 4, 1), ("f32", 8, 1)])
+def test_automatic_search_beyond_one_wave(kb, ctx, storage, k, flags):
+    """More tiles than the GPU holds at once, so that the automatic search keeps a tile to one CTA: value and
+    key lists over several chunks of the table."""
+    st = synth.small_stack(850 + k, 13, 330, 1300, K=5, nan_frac=0.01, n_angles=10, n_speeds=13, s_hi=80.0, n_sources=20,
+                           flux=60.0)
+    s = _stack(kb, ctx, st, storage)
+    if flags:   # rescored: the records of the FP32 planes' own candidates, in FP64
+        f = _stack(kb, ctx, st, "f32")
+        ctx.set_search_variant(4)
+        ref = _records(kb, ctx, f, st, 130, k, flags=kb.KB_RESCORE_FP64)
+        f.free()
+    else:
+        ctx.set_search_variant(5)
+        ref = _records(kb, ctx, s, st, 130, k)
+    ctx.set_search_variant(0)
+    assert _records(kb, ctx, s, st, 130, k, flags=kb.KB_RESCORE_FP64 if flags else 0).tobytes() == ref.tobytes()
+    s.free()
