@@ -13,8 +13,8 @@
 //     share the candidates of all of them, 32 at a time.  A thread per point
 //     walking linked lists spent its time in the dense groups around bright
 //     sources, one dependent load after the other: 262,144 candidates of a
-//     12 x 2048^2 search, core pass 1.92 -> 0.26 ms, unions 3.75 -> 0.32 ms, borders
-//     0.24 -> 0.17 ms;
+//     12 x 2048^2 search, core pass 1.92 -> 0.23 ms, unions 3.75 -> 0.32 ms, borders
+//     0.24 -> 0.09 ms;
 //   - distances are first taken in FP32, whose error is far below the margin it is
 //     given; only pairs within 2^-16 of eps take the FP64 distance (this GPU has two
 //     FP64 lanes per SM and cycle), and pairs already in one cluster take none;
